@@ -23,6 +23,7 @@ static uint64_t powmod(uint64_t b, uint64_t e, uint64_t q) {
     while (e) { if (e & 1) r = mulmod(r, b, q); b = mulmod(b, b, q); e >>= 1; }
     return r;
 }
+uint64_t pow_mod(uint64_t b, uint64_t e, uint64_t q) { return powmod(b, e, q); }
 uint64_t shoup_of(uint64_t w, uint64_t q) { return (uint64_t)(((u128)w << 64) / q); }
 
 // Deterministic Miller-Rabin for 64-bit integers (the first twelve primes as bases).
@@ -107,6 +108,7 @@ icm_ctx::~icm_ctx() {
     if (d_sdb_sgn) cudaFree(d_sdb_sgn);
     if (d_sq_pos) cudaFree(d_sq_pos);
     if (d_sq_sgn) cudaFree(d_sq_sgn);
+    nt.release();
     if (slot_tab) icm::free_slot_tables(slot_tab);
 }
 
@@ -303,6 +305,10 @@ icm_status icm_keygen(icm_ctx *c) {
     if (c->d_sdb_pos) { cudaFree(c->d_sdb_pos); cudaFree(c->d_sdb_sgn); cudaFree(c->d_sq_pos); cudaFree(c->d_sq_sgn); }
     c->d_sdb_pos = a; c->d_sdb_sgn = x; c->d_sq_pos = b; c->d_sq_sgn = y;
     c->max_db_blocks = max_blocks;
+    c->have_keys = false;
+    std::string why;
+    e = build_ntt(c, why);
+    if (e != cudaSuccess) return fail(ICM_ECUDA, "keygen transforms: " + (why.empty() ? cudaGetErrorString(e) : why));
     c->have_keys = true;
     // shared-memory opt-ins of the product kernels are set once here, outside any stream capture
     e = crt_set_attributes();

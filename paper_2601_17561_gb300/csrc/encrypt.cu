@@ -14,6 +14,8 @@
 //   where column j = eye * rho + r holds rotation r of the eye (Section 2.1.2).
 #include "icm_internal.h"
 
+#include <string>
+
 namespace {
 
 using icm::LayoutDev;
@@ -35,7 +37,7 @@ __device__ __forceinline__ int template_bit(const uint8_t *tpl, uint32_t b) { re
 
 struct DbMsgArgs {
     LayoutDev lay;
-    uint32_t K, d2, Nq, nqblk, h, code_bits, L, Lq;
+    uint32_t K, d2, Nq, nqblk, h, code_bits, Lq;
     const uint8_t *codes, *masks;      // [n_real][code_bits/8]
     const int32_t *wmsg;               // message rows [n_real][d2] (slot encoding), or null: c' of codes
     const int32_t *sq_pos; const int8_t *sq_sgn;   // [nqblk][h]
@@ -43,7 +45,8 @@ struct DbMsgArgs {
     uint64_t *db;                      // [L][M][K]
 };
 
-// Pass 1: the message residues Q' * W[r][k] of every stored b-row, for every limb.  The message
+// Pass 1: the message residues Q' * W[r][k] of every stored b-row, for the limbs of Q (they are zero
+// modulo the limbs of Q', which pass 2 does not read).  The message
 // row is the masked bit-vector c' of template r (coefficient encoding) or, for a slot-encoded
 // chunk, the given row of rounded slot-encoding coefficients.
 __global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
@@ -92,9 +95,9 @@ __global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
                 }
             }
         }
-        for (uint32_t l = 0; l < a.L; ++l) {
+        for (uint32_t l = 0; l < a.Lq; ++l) {
             uint64_t v = 0;
-            if (W != 0 && l < a.Lq) {
+            if (W != 0) {
                 const uint64_t m = mulmod_shoup((uint64_t)(W < 0 ? -W : W), a.qp[l], a.qps[l], a.q[l]);
                 v = (W < 0 && m) ? a.q[l] - m : m;
             }
@@ -105,118 +108,207 @@ __global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
 
 struct DbEncArgs {
     LayoutDev lay;
-    uint32_t K, h, eta, n_blocks;
+    uint32_t K, eta, n_blocks, Lq, logc;             // 2^logc columns per block
     uint64_t seed, chunk;
-    const int32_t *sdb_pos; const int8_t *sdb_sgn;   // [blocks][h]
+    icm::NttMod nt[ICM_MAX_LIMBS];
+    const uint64_t *shat;                            // [blocks][L][N]: transforms of s_{db,t}, times N^-1
     LimbTable lt;
     uint64_t *db;
 };
 
-// Pass 2, one block per (column k, limb l): draw the a-part column into shared memory and write
-// it, then finish every b-row: B = msg - (s_{db,t} * a)[i] + e (mod q_l).
-__global__ void __launch_bounds__(1024) k_db_apart_b(DbEncArgs a) {
-    extern __shared__ unsigned char smem[];
-    uint64_t *acol = reinterpret_cast<uint64_t *>(smem);                 // [N]
-    int32_t *spos = reinterpret_cast<int32_t *>(acol + a.lay.N);         // [n_blocks*h]
-    int8_t *ssgn = reinterpret_cast<int8_t *>(spos + a.n_blocks * a.h);
+// Threads of the kernels that multiply by a secret: 128 registers each, of which a thread keeps
+// up to 32 words of a transformed polynomial.
+constexpr int NT_MUL = 512;
 
-    const uint32_t k = blockIdx.x, l = blockIdx.y, N = a.lay.N;
+// Pass 2, one block per (2^logc columns k, limb l): draw the a-part columns into shared memory and
+// write them, then finish every b-row: B = msg - (s_{db,t} * a)[i] + e (mod q_l).
+//
+// The products by the secrets are negacyclic transforms (ntt.cuh): one forward transform of a, which
+// stays in registers, and per block t a pointwise product and one inverse transform.  Integer
+// arithmetic bounds both this and the direct form (h = 512 modular additions per coefficient),
+// but a transform costs about 7 Shoup products per coefficient.  Columns are taken four at a time
+// where 2^14 words hold them, so that a row's words fill a 32-byte sector and the columns share
+// their twiddles.  1,000 templates at N_db = 2^12, four primes (4.0 GB): 69.5 ms with the
+// additions, 15.3 ms now.
+template <int WPT>
+__global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant__ DbEncArgs a) {
+    extern __shared__ uint64_t su[];                                     // [2^logc][stride]
+    const uint32_t C = 1u << a.logc, l = blockIdx.y, N = a.lay.N, k0 = blockIdx.x << a.logc;
+    const uint32_t stride = icm::ntt_words(N) + 4, CN = N << a.logc;
     const uint64_t q = a.lt.q[l];
+    const icm::NttMod &T = a.nt[l];
     const uint64_t ka = stream_key(a.seed, ICM_KIND_A_DB, a.chunk, l);
     const uint64_t ke = stream_key(a.seed, ICM_KIND_E_DB, a.chunk, 0);
     uint64_t *dbl = a.db + (size_t)l * a.lay.M * a.K;
-    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
-        const uint64_t v = uniform_mod(sm64(ka, (uint64_t)i * a.K + k), q);
-        acol[i] = v;
-        dbl[(size_t)i * a.K + k] = to_digit_form(v, q);
-    }
-    for (uint32_t x = threadIdx.x; x < a.n_blocks * a.h; x += blockDim.x) { spos[x] = a.sdb_pos[x]; ssgn[x] = a.sdb_sgn[x]; }
-    __syncthreads();
-
-    const uint64_t nb = a.lay.M - N;
-    for (uint64_t bidx = threadIdx.x; bidx < nb; bidx += blockDim.x) {
-        uint32_t t, i;
-        b_row_of(a.lay, bidx, t, i);
-        const uint64_t r = (uint64_t)t * N + i;
-        uint64_t sa = 0;       // (s_{db,t} * a)[i] mod q
-        for (uint32_t c = 0; c < a.h; ++c) {
-            const uint32_t p = (uint32_t)spos[t * a.h + c];
-            const int s = ssgn[t * a.h + c];
-            // X^p * X^(i-p): wraps with a sign flip when i < p
-            const uint64_t term = (i >= p) ? acol[i - p] : acol[N + i - p];
-            const bool neg = (i >= p) ? (s < 0) : (s > 0);
-            sa = neg ? sub_mod(sa, term, q) : add_mod(sa, term, q);
+    // word x: column x mod C of coefficient x / C
+    for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
+        const uint32_t c = x & (C - 1), i = x >> a.logc, k = k0 + c;
+        uint64_t v = 0;
+        if (k < a.K) {
+            v = uniform_mod(sm64(ka, (uint64_t)i * a.K + k), q);
+            dbl[(size_t)i * a.K + k] = to_digit_form(v, q);
         }
-        uint64_t *dst = dbl + (size_t)(N + bidx) * a.K + k;
-        const int e = cbd_sample(sm64(ke, r * a.K + k), a.eta);
-        uint64_t v = sub_mod(*dst, sa, q);
-        v = e >= 0 ? add_mod(v, (uint64_t)e, q) : sub_mod(v, (uint64_t)(-e), q);
-        *dst = to_digit_form(v, q);
+        su[c * stride + icm::ntt_pad(i)] = v;
+    }
+    if (a.n_blocks == 0) return;
+    __syncthreads();
+    icm::ntt_forward(su, C, stride, N, T);
+    uint64_t ah[WPT];
+#pragma unroll
+    for (int j = 0; j < WPT; ++j) {
+        const uint32_t x = threadIdx.x + j * NT_MUL;
+        if (x < CN) ah[j] = su[(x & (C - 1)) * stride + icm::ntt_pad(x >> a.logc)];
+    }
+    for (uint32_t t = 0; t < a.n_blocks; ++t) {
+        // a thread overwrites only the words that it read itself
+        const uint64_t *sh = a.shat + ((size_t)t * a.lt.n + l) * N;
+#pragma unroll
+        for (int j = 0; j < WPT; ++j) {
+            const uint32_t x = threadIdx.x + j * NT_MUL;
+            if (x < CN)
+                su[(x & (C - 1)) * stride + icm::ntt_pad(x >> a.logc)] = icm::mul_r128_lazy(ah[j], __ldg(sh + (x >> a.logc)), T);
+        }
+        __syncthreads();
+        icm::ntt_inverse(su, C, stride, N, T);
+        const bool part = t >= a.lay.n_full;                             // the partial last block
+        for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
+            const uint32_t c = x & (C - 1), i = x >> a.logc, k = k0 + c;
+            if (k >= a.K || (part && i >= a.lay.rem && i < a.lay.tail_lo)) continue;
+            const uint64_t row = (uint64_t)N + (uint64_t)t * N + (part && i >= a.lay.rem ? a.lay.rem + (i - a.lay.tail_lo) : i);
+            const uint64_t r = (uint64_t)t * N + i;
+            uint64_t sa = su[c * stride + icm::ntt_pad(i)];              // (s_{db,t} * a)[i], below 2q
+            sa = sa >= q ? sa - q : sa;
+            uint64_t *dst = dbl + (size_t)row * a.K + k;
+            const int e = cbd_sample(sm64(ke, r * a.K + k), a.eta);
+            // messages are multiples of Q', zero modulo the limbs of Q'
+            uint64_t v = sub_mod(l < a.Lq ? *dst : 0, sa, q);
+            v = e >= 0 ? add_mod(v, (uint64_t)e, q) : sub_mod(v, (uint64_t)(-e), q);
+            *dst = to_digit_form(v, q);
+        }
     }
 }
 
 struct QEncArgs {
-    uint32_t K, d2, Nq, h, eta, rho, code_bits, Lq, nqblk;
+    uint32_t K, d2, Nq, eta, rho, code_bits, Lq, nqblk, logc;            // 2^logc columns per block
     uint64_t seed;
     const uint8_t *codes, *masks;        // [n_eyes][code_bits/8]
     const uint64_t *eye_ids;
-    const int32_t *sq_pos; const int8_t *sq_sgn;
+    icm::NttMod nt[2];
+    const uint64_t *shat;                // [nqblk][Lq][Nq]: transforms of s_{q,t}, times Nq^-1
     uint64_t q[ICM_MAX_LIMBS], dl[ICM_MAX_LIMBS];   // primes and Delta mod q_l
     uint32_t n_cols;
     uint64_t *ct;                        // [Lq][n_cols][K]
 };
 
-// One block per (query column j, limb l < Lq).
-__global__ void __launch_bounds__(1024) k_query_encrypt(QEncArgs a) {
-    extern __shared__ unsigned char smem[];
-    uint64_t *acol = reinterpret_cast<uint64_t *>(smem);           // [Nq]
-    int8_t *cp = reinterpret_cast<int8_t *>(acol + a.Nq);          // [d2]
-    const uint32_t j = blockIdx.x, l = blockIdx.y;
-    const uint32_t e = j / a.rho, r = j % a.rho;
-    const int shift = (int)r - (int)(a.rho - 1) / 2;
+// One block per (2^logc query columns, limb l < Lq): the same transforms as k_db_apart_b.  32 eyes
+// (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient,
+// 1.26 ms now.
+template <int WPT>
+__global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_constant__ QEncArgs a) {
+    extern __shared__ uint64_t su[];                               // [2^logc][stride]
+    const uint32_t C = 1u << a.logc, l = blockIdx.y, N = a.Nq, j0 = blockIdx.x << a.logc;
+    const uint32_t stride = icm::ntt_words(N) + 4, CN = N << a.logc;
     const uint64_t q = a.q[l];
-    const uint64_t eid = a.eye_ids[e];
-    const uint64_t ka = stream_key(a.seed, ICM_KIND_A_Q, eid, l);
-    const uint64_t ke = stream_key(a.seed, ICM_KIND_E_Q, eid, 0);
-    uint64_t *col = a.ct + ((size_t)l * a.n_cols + j) * a.K;
-    const uint32_t tb = a.code_bits / 8;
-    const uint8_t *cd = a.codes + (size_t)e * tb, *mk = a.masks + (size_t)e * tb;
-    // rotated masked bit-vector: x_s[row, col, b] = x[row, (col + s) mod 200, b] on 16 x 200 x 4
-    for (uint32_t k = threadIdx.x; k < a.d2; k += blockDim.x) {
-        int v = 0;
-        if (k < a.code_bits) {
-            const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
-            const uint32_t src_col = (uint32_t)(((int)cc + shift + 200) % 200);
-            const uint32_t src = (row * 200 + src_col) * 4 + b;
-            const int c = template_bit(cd, src), m = template_bit(mk, src);
-            v = m - 2 * (c & m);
+    const icm::NttMod &T = a.nt[l];
+    // word x: coefficient x mod N of column x / N
+    for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
+        const uint32_t c = x / N, i = x % N, j = j0 + c;
+        uint64_t v = 0;
+        if (j < a.n_cols) {
+            const uint64_t ka = stream_key(a.seed, ICM_KIND_A_Q, a.eye_ids[j / a.rho], l);
+            v = uniform_mod(sm64(ka, (uint64_t)(j % a.rho) * N + i), q);
+            a.ct[((size_t)l * a.n_cols + j) * a.K + a.d2 + i] = v;
         }
-        cp[k] = (int8_t)v;
-    }
-    for (uint32_t i = threadIdx.x; i < a.Nq; i += blockDim.x) {
-        const uint64_t v = uniform_mod(sm64(ka, (uint64_t)r * a.Nq + i), q);
-        acol[i] = v;
-        col[a.d2 + i] = v;
+        su[c * stride + icm::ntt_pad(i)] = v;
     }
     __syncthreads();
-    for (uint32_t k = threadIdx.x; k < a.d2; k += blockDim.x) {
-        const uint32_t t = k / a.Nq, i = k % a.Nq;
-        uint64_t sa = 0;
-        for (uint32_t c = 0; c < a.h; ++c) {
-            const uint32_t p = (uint32_t)a.sq_pos[t * a.h + c];
-            const int s = a.sq_sgn[t * a.h + c];
-            const uint64_t term = (i >= p) ? acol[i - p] : acol[a.Nq + i - p];
-            const bool neg = (i >= p) ? (s < 0) : (s > 0);
-            sa = neg ? sub_mod(sa, term, q) : add_mod(sa, term, q);
-        }
-        uint64_t v = sa ? q - sa : 0;                          // -(s * a)
-        const int m = cp[k];
-        if (m > 0) v = add_mod(v, a.dl[l], q);
-        else if (m < 0) v = sub_mod(v, a.dl[l], q);
-        const int err = cbd_sample(sm64(ke, (uint64_t)r * a.d2 + k), a.eta);
-        v = err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
-        col[k] = v;
+    icm::ntt_forward(su, C, stride, N, T);
+    uint64_t ah[WPT];
+#pragma unroll
+    for (int w = 0; w < WPT; ++w) {
+        const uint32_t x = threadIdx.x + w * NT_MUL;
+        if (x < CN) ah[w] = su[(x / N) * stride + icm::ntt_pad(x % N)];
     }
+    const uint32_t tb = a.code_bits / 8;
+    for (uint32_t t = 0; t < a.nqblk; ++t) {
+        const uint64_t *sh = a.shat + ((size_t)t * a.Lq + l) * N;
+#pragma unroll
+        for (int w = 0; w < WPT; ++w) {
+            const uint32_t x = threadIdx.x + w * NT_MUL;
+            if (x < CN)
+                su[(x / N) * stride + icm::ntt_pad(x % N)] = icm::mul_r128_lazy(ah[w], __ldg(sh + x % N), T);
+        }
+        __syncthreads();
+        icm::ntt_inverse(su, C, stride, N, T);
+        for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
+            const uint32_t c = x / N, i = x % N, j = j0 + c, k = t * N + i;
+            if (j >= a.n_cols) continue;
+            const uint32_t e = j / a.rho, r = j % a.rho;
+            uint64_t sa = su[c * stride + icm::ntt_pad(i)];
+            sa = sa >= q ? sa - q : sa;
+            uint64_t v = sa ? q - sa : 0;                          // -(s * a)
+            // rotated masked bit-vector: x_s[row, col, b] = x[row, (col + s) mod 200, b] on 16 x 200 x 4
+            int m = 0;
+            if (k < a.code_bits) {
+                const int shift = (int)r - (int)(a.rho - 1) / 2;
+                const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
+                const uint32_t src = (row * 200 + (uint32_t)(((int)cc + shift + 200) % 200)) * 4 + b;
+                const int cb = template_bit(a.codes + (size_t)e * tb, src), mb = template_bit(a.masks + (size_t)e * tb, src);
+                m = mb - 2 * (cb & mb);
+            }
+            if (m > 0) v = add_mod(v, a.dl[l], q);
+            else if (m < 0) v = sub_mod(v, a.dl[l], q);
+            const uint64_t ke = stream_key(a.seed, ICM_KIND_E_Q, a.eye_ids[e], 0);
+            const int err = cbd_sample(sm64(ke, (uint64_t)r * a.d2 + k), a.eta);
+            v = err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
+            a.ct[((size_t)l * a.n_cols + j) * a.K + k] = v;
+        }
+    }
+}
+
+// Transform tables of one modulus (icm_internal.h): entry k of [0, N) is psi^bitrev(k), then psi^-1.
+struct TabArgs {
+    uint32_t N, logN;
+    uint64_t psi, ipsi;
+    icm::NttMod T;
+    ulonglong2 *out;                     // [2][N]
+};
+__device__ __forceinline__ uint64_t mul_exact(uint64_t a, uint64_t b, const icm::NttMod &T) {
+    const uint64_t r = icm::mul_r128_lazy(a, b, T);
+    return r >= T.q ? r - T.q : r;
+}
+__global__ void k_ntt_table(const __grid_constant__ TabArgs a) {
+    const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
+    if (x >= 2 * a.N) return;
+    uint32_t e = __brev(x & (a.N - 1)) >> (32 - a.logN);
+    uint64_t b = x >= a.N ? a.ipsi : a.psi, w = 1;
+    for (; e; e >>= 1, b = mul_exact(b, b, a.T))
+        if (e & 1) w = mul_exact(w, b, a.T);
+    // floor(w 2^64 / q): the estimate from floor(2^128 / q) is short by at most one
+    uint64_t ws = w * a.T.rhi + __umul64hi(w, a.T.rlo);
+    if ((uint64_t)0 - ws * a.T.q >= a.T.q) ++ws;
+    a.out[x] = make_ulonglong2(w, ws);
+}
+
+// Transforms of the sparse secrets, times N^-1: one block per (secret t, limb l).
+struct SecArgs {
+    uint32_t N, h, L;
+    icm::NttMod nt[ICM_MAX_LIMBS];
+    const int32_t *pos; const int8_t *sgn;           // [t][h]
+    uint64_t *out;                                   // [t][L][N]
+};
+__global__ void __launch_bounds__(NT_MUL, 1) k_ntt_secret(const __grid_constant__ SecArgs a) {
+    extern __shared__ uint64_t su[];
+    const uint32_t t = blockIdx.x, l = blockIdx.y;
+    const icm::NttMod &T = a.nt[l];
+    for (uint32_t i = threadIdx.x; i < icm::ntt_words(a.N); i += NT_MUL) su[i] = 0;
+    __syncthreads();
+    for (uint32_t c = threadIdx.x; c < a.h; c += NT_MUL)
+        su[icm::ntt_pad((uint32_t)a.pos[t * a.h + c])] = a.sgn[t * a.h + c] < 0 ? T.q - 1 : 1;
+    __syncthreads();
+    icm::ntt_forward(su, 1, 0, a.N, T);
+    for (uint32_t i = threadIdx.x; i < a.N; i += NT_MUL)
+        a.out[((size_t)t * a.L + l) * a.N + i] = mulmod_shoup(su[icm::ntt_pad(i)], T.ninv, T.ninvs, T.q);
 }
 
 }  // namespace
@@ -228,10 +320,10 @@ cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uin
     DbMsgArgs a{};
     a.lay = lay;
     a.K = c->K; a.d2 = c->p.d2; a.Nq = c->N_q; a.nqblk = c->n_qblk; a.h = c->p.hamming_weight;
-    a.code_bits = c->p.code_bits; a.L = c->p.n_limbs; a.Lq = c->p.n_limbs_q;
+    a.code_bits = c->p.code_bits; a.Lq = c->p.n_limbs_q;
     a.codes = d_codes; a.masks = d_masks; a.wmsg = d_wmsg;
     a.sq_pos = c->d_sq_pos; a.sq_sgn = c->d_sq_sgn;
-    for (uint32_t l = 0; l < a.L; ++l) { a.qp[l] = c->qp_mod[l]; a.qps[l] = c->qp_mods[l]; a.q[l] = c->q[l]; }
+    for (uint32_t l = 0; l < a.Lq; ++l) { a.qp[l] = c->qp_mod[l]; a.qps[l] = c->qp_mods[l]; a.q[l] = c->q[l]; }
     a.db = d_db;
     const uint64_t nb = lay.M - lay.N;
     if (nb == 0) return cudaSuccess;
@@ -242,39 +334,111 @@ cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uin
     return cudaGetLastError();
 }
 
+// Columns per block of the secret-product kernels: as many as 2^14 words hold, at most `want`.
+static uint32_t mul_logc(uint32_t N, uint32_t want) {
+    uint32_t lc = 0;
+    while ((2u << lc) <= want && ((uint64_t)N << (lc + 1)) <= 16384) ++lc;
+    return lc;
+}
+static size_t mul_smem(uint32_t N, uint32_t logc) { return ((size_t)(ntt_words(N) + 4) << logc) * 8; }
+
+template <typename K, typename A>
+static cudaError_t launch_mul(K kern, const A &a, dim3 grid, size_t smem, cudaStream_t st) {
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kern<<<grid, NT_MUL, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_db_apart_and_b(const icm_ctx *c, const LayoutDev &lay, uint64_t chunk_id, uint64_t *d_db,
                                   cudaStream_t st) {
+    if (!c->nt.shat_db) return cudaErrorInvalidValue;                    // rings above 2^14
     DbEncArgs a{};
-    a.lay = lay; a.K = c->K; a.h = c->p.hamming_weight; a.eta = c->p.noise_eta;
+    a.lay = lay; a.K = c->K; a.eta = c->p.noise_eta; a.Lq = c->p.n_limbs_q;
     a.n_blocks = (uint32_t)((lay.M - lay.N) ? (lay.n_full + (lay.rem ? 1 : 0)) : 0);
     a.seed = c->p.seed; a.chunk = chunk_id;
-    a.sdb_pos = c->d_sdb_pos; a.sdb_sgn = c->d_sdb_sgn;
+    a.logc = mul_logc(lay.N, 4);
+    for (uint32_t l = 0; l < c->p.n_limbs; ++l) a.nt[l] = c->nt.db[l];
+    a.shat = c->nt.shat_db;
     a.lt = c->lt; a.db = d_db;
-    const size_t smem = (size_t)lay.N * 8 + (size_t)a.n_blocks * a.h * 5;
-    cudaError_t e = cudaFuncSetAttribute(k_db_apart_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(c->K, c->p.n_limbs);
-    k_db_apart_b<<<grid, 1024, smem, st>>>(a);
-    return cudaGetLastError();
+    const size_t smem = mul_smem(lay.N, a.logc);
+    dim3 grid((c->K + (1u << a.logc) - 1) >> a.logc, c->p.n_limbs);
+    const uint32_t wpt = (uint32_t)(((uint64_t)lay.N << a.logc) + NT_MUL - 1) / NT_MUL;
+    return wpt > 16 ? launch_mul(k_db_apart_b<32>, a, grid, smem, st)
+                    : wpt > 8 ? launch_mul(k_db_apart_b<16>, a, grid, smem, st) : launch_mul(k_db_apart_b<8>, a, grid, smem, st);
 }
 
 cudaError_t launch_query_encrypt(const icm_ctx *c, const uint8_t *d_codes, const uint8_t *d_masks,
                                  const uint64_t *d_eye_ids, uint32_t n_eyes, uint64_t *d_ct, cudaStream_t st) {
     QEncArgs a{};
-    a.K = c->K; a.d2 = c->p.d2; a.Nq = c->N_q; a.h = c->p.hamming_weight; a.eta = c->p.noise_eta;
+    a.K = c->K; a.d2 = c->p.d2; a.Nq = c->N_q; a.eta = c->p.noise_eta;
     a.rho = c->p.rho; a.code_bits = c->p.code_bits; a.Lq = c->p.n_limbs_q; a.nqblk = c->n_qblk;
     a.seed = c->p.seed; a.codes = d_codes; a.masks = d_masks; a.eye_ids = d_eye_ids;
-    a.sq_pos = c->d_sq_pos; a.sq_sgn = c->d_sq_sgn;
-    for (uint32_t l = 0; l < a.Lq; ++l) { a.q[l] = c->q[l]; a.dl[l] = c->delta_mod[l]; }
+    for (uint32_t l = 0; l < a.Lq; ++l) { a.q[l] = c->q[l]; a.dl[l] = c->delta_mod[l]; a.nt[l] = c->nt.q[l]; }
+    a.shat = c->nt.shat_q;
     a.n_cols = n_eyes * c->p.rho;
     a.ct = d_ct;
     if (a.n_cols == 0) return cudaSuccess;
-    const size_t smem = (size_t)a.Nq * 8 + a.d2;
-    cudaError_t e = cudaFuncSetAttribute(k_query_encrypt, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(a.n_cols, a.Lq);
-    k_query_encrypt<<<grid, 1024, smem, st>>>(a);
-    return cudaGetLastError();
+    if (!a.shat) return cudaErrorInvalidValue;                           // rings above 2^14
+    // two columns share their twiddles where there are enough of them to fill the SMs
+    a.logc = mul_logc(a.Nq, a.n_cols * a.Lq >= 2 * 152 ? 2 : 1);
+    const size_t smem = mul_smem(a.Nq, a.logc);
+    dim3 grid((a.n_cols + (1u << a.logc) - 1) >> a.logc, a.Lq);
+    const uint32_t wpt = ((a.Nq << a.logc) + NT_MUL - 1) / NT_MUL;
+    return wpt > 16 ? launch_mul(k_query_encrypt<32>, a, grid, smem, st)
+                    : wpt > 8 ? launch_mul(k_query_encrypt<16>, a, grid, smem, st)
+                              : launch_mul(k_query_encrypt<8>, a, grid, smem, st);
+}
+
+// Builds the transform tables and the secrets' transforms (icm_keygen, after the supports are on the
+// device).  Rings above 2^14 have no secret-product kernels and get no tables.
+cudaError_t build_ntt(icm_ctx *c, std::string &why) {
+    NttSet &S = c->nt;
+    S.release();
+    const uint32_t rings[2] = {c->N_db, c->N_q}, limbs[2] = {c->p.n_limbs, c->p.n_limbs_q};
+    const uint32_t secrets[2] = {c->max_db_blocks, c->n_qblk};
+    for (int w = 0; w < 2; ++w) {
+        const uint32_t N = rings[w], L = limbs[w];
+        if (N > 16384) continue;
+        uint32_t logN = 0;
+        while ((1u << logN) < N) ++logN;
+        ulonglong2 **tab = w ? &S.tab_q : &S.tab_db;
+        uint64_t **shat = w ? &S.shat_q : &S.shat_db;
+        NttMod *nt = w ? S.q : S.db;
+        cudaError_t e = cudaMalloc(tab, (size_t)L * 2 * N * sizeof(ulonglong2));
+        if (e != cudaSuccess) return e;
+        for (uint32_t l = 0; l < L; ++l) {
+            const uint64_t q = c->q[l];
+            if ((q - 1) % (2ull * N)) { why = "primes must be 1 mod 2 N"; return cudaErrorInvalidValue; }
+            // psi: a primitive 2N-th root of unity, g^((q-1)/2N) for a quadratic non-residue g
+            uint64_t psi = 0;
+            for (uint64_t g = 2; g < 1000 && !psi; ++g)
+                if (pow_mod(g, (q - 1) / 2, q) == q - 1) psi = pow_mod(g, (q - 1) / (2ull * N), q);
+            if (!psi || pow_mod(psi, N, q) != q - 1) { why = "no primitive 2N-th root"; return cudaErrorInvalidValue; }
+            NttMod &m = nt[l];
+            m.q = q;
+            m.ninv = pow_mod(N, q - 2, q); m.ninvs = shoup_of(m.ninv, q);
+            m.rhi = c->crt.rhi[l]; m.rlo = c->crt.rlo[l];
+            m.fwd = *tab + (size_t)l * 2 * N; m.inv = m.fwd + N;
+            TabArgs a{N, logN, psi, pow_mod(psi, q - 2, q), m, *tab + (size_t)l * 2 * N};
+            k_ntt_table<<<(2 * N + 255) / 256, 256>>>(a);
+        }
+        e = cudaMalloc(shat, (size_t)secrets[w] * L * N * 8);
+        if (e != cudaSuccess) return e;
+        SecArgs a{};
+        a.N = N; a.h = c->p.hamming_weight; a.L = L;
+        for (uint32_t l = 0; l < L; ++l) a.nt[l] = nt[l];
+        a.pos = w ? c->d_sq_pos : c->d_sdb_pos; a.sgn = w ? c->d_sq_sgn : c->d_sdb_sgn;
+        a.out = *shat;
+        e = launch_mul(k_ntt_secret, a, dim3(secrets[w], L), (size_t)ntt_words(N) * 8, nullptr);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaStreamSynchronize(nullptr);
+}
+
+void NttSet::release() {
+    cudaFree(tab_db); cudaFree(tab_q); cudaFree(shat_db); cudaFree(shat_q);
+    *this = NttSet{};
 }
 
 }  // namespace icm

@@ -9,6 +9,7 @@
 
 #include "../../include/icm.h"
 #include "icm_device.cuh"
+#include "ntt.cuh"
 #include "ppmm_i8.h"
 
 namespace icm {
@@ -40,6 +41,15 @@ struct RescaleConsts {
     uint64_t qp[ICM_MAX_LIMBS], qps[ICM_MAX_LIMBS], qpinv[ICM_MAX_LIMBS], qpinvs[ICM_MAX_LIMBS];
 };
 
+// Transforms of the rings up to 2^14 (ntt.cuh), on the context's device: tables per limb, and the
+// secrets' transforms [t][limbs][N] times N^-1.
+struct NttSet {
+    NttMod db[ICM_MAX_LIMBS] = {}, q[2] = {};
+    ulonglong2 *tab_db = nullptr, *tab_q = nullptr;
+    uint64_t *shat_db = nullptr, *shat_q = nullptr;
+    void release();
+};
+
 }  // namespace icm
 
 namespace icm { struct SlotTables; void free_slot_tables(SlotTables *t); }
@@ -65,6 +75,7 @@ struct icm_ctx {
     uint32_t max_db_blocks = 0;
     int32_t *d_sdb_pos = nullptr;  int8_t *d_sdb_sgn = nullptr;   // [max_db_blocks][h]
     int32_t *d_sq_pos = nullptr;   int8_t *d_sq_sgn = nullptr;    // [n_qblk][h]
+    icm::NttSet nt;                        // transforms of the rings and secrets (icm_keygen)
     icm::SlotTables *slot_tab = nullptr;   // slot-encoding and NTT tables (built on first use)
     ~icm_ctx();
 };
@@ -138,6 +149,8 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
 // Rescaling by Q' of n coefficients per limb: [L][n] at modulus Q_db -> [L_q][n] at modulus Q.
 cudaError_t launch_rescale(const icm_ctx *c, const uint64_t *d_in, uint64_t n, uint64_t *d_out, cudaStream_t st);
 
+cudaError_t build_ntt(icm_ctx *c, std::string &why);
+uint64_t pow_mod(uint64_t b, uint64_t e, uint64_t q);
 LimbTable make_limb_table(const std::vector<uint64_t> &q);
 uint64_t shoup_of(uint64_t w, uint64_t q);
 

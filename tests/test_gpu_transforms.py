@@ -1,0 +1,43 @@
+"""The encryption kernels' products by the secrets (negacyclic transforms) at the edges of their range: the
+smallest rings, one, two and four columns per block, partial blocks, two query primes, against the
+oracle bit by bit."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+from paper_2601_17561_gb300 import build as B
+from paper_2601_17561_gb300 import engine as E
+from paper_2601_17561_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+# (log N_db, log N_q, limbs, query limbs, templates, eyes): N_db = 32 with rho = 31 and several blocks; sizes
+# that leave one transform level over a multiple of three, two and none; N_q = 2^14 (one column per block)
+SHAPES = [(5, 5, 2, 1, 70, 1), (7, 14, 3, 1, 300, 2), (9, 9, 2, 1, 40, 12), (11, 13, 4, 2, 30, 6)]
+
+
+def _u64(t, shape):
+    n = int(np.prod(shape))
+    return t[: n * 8].view(torch.int64).cpu().numpy().view(np.uint64).reshape(shape)
+
+
+def _from_digit_form(z, q):
+    B8 = np.uint64(0x8080808080808080)
+    c = ((z ^ B8) - B8).view(np.int64)
+    return np.stack([np.where(c[i] < 0, c[i] + np.int64(ql), c[i]).view(np.uint64) for i, ql in enumerate(q)])
+
+
+@pytest.mark.parametrize("log_n_db,log_n_q,L,Lq,n_db,n_eyes", SHAPES)
+def test_encryption_ring_edges(log_n_db, log_n_q, L, Lq, n_db, n_eyes):
+    B.build()
+    prm = dict(log_n_db=log_n_db, log_n_q=log_n_q, n_limbs=L, n_limbs_q=Lq, prime_bits=60,
+               log2_delta=60 if Lq == 2 else 40, seed=9)
+    P = O.Params(**prm, h=16)
+    W = synth.make_workload(n_eyes=n_eyes, n_db=n_db, seed=21)
+    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    ct = O.query_encrypt(P, W.q_codes, W.q_masks, W.eye_ids)
+    assert np.array_equal(_u64(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), ct.shape), ct)
+    A = O.db_rows(P, W.db_codes, W.db_masks, O.db_layout(n_db, P.ndb, P.rho))
+    db = eng.encrypt_db(W.db_codes, W.db_masks)
+    assert np.array_equal(_from_digit_form(_u64(db.buf, A.shape), P.q), A)
