@@ -274,7 +274,7 @@ icm_status icm_match_batch_workspace_bytes(const icm_ctx *ctx, const icm_db *con
 /* CCMM of one prepared query batch against 1..16 database chunks (each its own MSRLWE database
  * with its own a-part, uneven sizes allowed; Section 6.2.3 distributes the database the same way
  * over GPUs).  For the CRT forms every limb, chunk, row tile, modulus and column tile of a round of
- * up to 512 columns is one persistent kernel launch; the u64 and digit forms launch per chunk.
+ * up to 1,024 columns (512 on mma.sync) is one persistent kernel launch; the u64 and digit forms launch per chunk.
  * dev_outs[i]: scores of chunk i (icm_scores_bytes of that chunk); outs[i] receives its handle. */
 icm_status icm_match_batch(icm_ctx *ctx, const icm_db *const *dbs, size_t n_dbs, const icm_query *q,
                            void *const *dev_outs, const size_t *out_bytes, void *dev_ws, size_t ws_bytes, void *stream,
@@ -294,20 +294,20 @@ void icm_plan_destroy(icm_plan *plan);
 
 /* Kernel variant of the CRT forms' product: 256 = mma.sync with 256-column tiles, 128 = mma.sync
  * with 128-column tiles; for the fp16 form on a database in the storage form, the tcgen05 kernel
- * (tensor-memory accumulators, TMA-fed, one modulus on 512 columns per block and round, every
- * round of up to 1,024 columns in one launch; needs an even K, else variant 256 runs): 1 = rings
- * of 8 raw-database and 4 operand slots; 2 = the same with a wave bound between blocks (a block
- * starts fetching its next tile once every block has fetched its current one; cooperative
- * launch); 3 = 4 raw-database and 8 operand slots.  0 restores the default, variant 2 (which the
- * int8 form and odd K run as 256).  Results are identical; only speed differs. */
+ * (block pairs with tensor-memory accumulators: 128 database rows x up to 1,024 columns of one
+ * modulus, or several moduli of fewer columns, per pair; needs an even K, else variant 256 runs):
+ * 1 = free-running pairs; 2 = with a wave bound between pairs (a pair starts fetching its next tile
+ * once every pair has fetched its current one; cooperative launch) and the moduli in groups of six;
+ * 3 = with the wave bound and all moduli of a row tile side by side.  0 restores the default,
+ * variant 2 (which the int8 form and odd K run as 256).  Results are identical; only speed differs. */
 icm_status icm_ctx_set_variant(icm_ctx *ctx, int variant);
 /* Failure detection of the tcgen05 kernel (no counterpart in the paper).  Every device-side wait
  * of that kernel (barrier phases, the wave bound) gives up after wait_ns nanoseconds of
  * %globaltimer (0 restores the default, 2 s): the kernel then records ICM_ETIMEOUT in the device
  * status word, stops issuing work, waits (bounded) for its own copies and MMAs in flight, frees
  * its tensor memory and returns; its outputs are then invalid.  inject_stall != 0 is for tests
- * only: the kernel's query producer of the first column tile then issues no copies, so the MMA
- * issuer's wait runs out on purpose (no fault, no trap).  Applies to later launches from this
+ * only: the kernel's query producers then issue no copies, so the MMA issuer's wait runs out on
+ * purpose (no fault, no trap).  Applies to later launches from this
  * context.  Errors: ICM_EINVAL for a null context. */
 icm_status icm_ctx_set_device_wait(icm_ctx *ctx, uint64_t wait_ns, int inject_stall);
 /* Device status word shared by the library's kernels: ICM_OK, or ICM_ETIMEOUT once a kernel gave

@@ -183,7 +183,7 @@ __global__ void __launch_bounds__(NT, 1) k_crt_p1(P1Args p) {
         for (int e = 0; e < (BN * CH) / NT; ++e) {
             const int idx = tid + e * NT, col = idx / CH, ch = idx % CH;
             const bool ok = p.n0 + nb + col < N && nb + col < p.nch;
-            const uint64_t off = F16 ? icm::crt_f16_off(p.n0 + nb + col, k0 + ch * 8, Kp) * 2
+            const uint64_t off = F16 ? icm::crt_f16_off(p.n0 + nb + col, k0 + ch * 8, N, Kp) * 2
                                      : ((nb + col) * Kp + k0) * ESZ + ch * 16;
             const unsigned char *src = Bl + (ok ? off : 0);
             cp_async16(smem_u32(sB + (size_t)st * BN * LDB + col * LDB + ch * 16), src, ok);
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(256) k_crt_planes_f16(const uint64_t *op, __ha
         uint64_t v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) v[e] = (j < N && k0 + e < K) ? op[((size_t)l * N + j) * K + k0 + e] : 0;
-        const uint64_t o = icm::crt_f16_off(j, k0, Kp);
+        const uint64_t o = icm::crt_f16_off(j, k0, N, Kp);
         for (uint32_t i = 0; i < r; ++i) {
             uint32_t w[4];
 #pragma unroll

@@ -21,10 +21,6 @@ struct I8Consts {
     int32_t mod[ICM_MAX_MODULI], wlo[ICM_MAX_MODULI], whi[ICM_MAX_MODULI], yinv[ICM_MAX_MODULI];
     float inv_m[ICM_MAX_MODULI];
     uint32_t r19[ICM_MAX_MODULI];
-    // integer residue conversion of the tcgen05 path: dp4a bias c = m ceil(2^17 / m) + h with
-    // h = floor(m / 2), division magic ceil(2^32 / m), and the f16x2 bits of -(1024 + h)
-    int32_t cbias[ICM_MAX_MODULI];
-    uint32_t magic[ICM_MAX_MODULI], hneg2[ICM_MAX_MODULI];
     uint64_t W[ICM_MAX_LIMBS][ICM_MAX_MODULI], Ws[ICM_MAX_LIMBS][ICM_MAX_MODULI], Wy[ICM_MAX_LIMBS][ICM_MAX_MODULI];
     uint64_t Mq[ICM_MAX_LIMBS], Mqs[ICM_MAX_LIMBS];
     // p^2 form: q_l = pd_l^2, digit base pd_l and 1 / pd_l (pw8[l][0..1] hold 1 and pd_l)
@@ -61,9 +57,9 @@ cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const C
                                     uint64_t K, uint64_t Kp, void *scratch, cudaStream_t st);
 cudaError_t crt_set_attributes();
 // Kernel variants of the CRT product: the column tile of the mma.sync kernel (128, 256), or the
-// tcgen05 kernel for the fp16 form on the balanced-digit database (one launch per 1,024 columns):
-// 1 = rings of 8 raw-database and 4 operand slots, 2 = the same with the wave bound between blocks
-// (cooperative launch), 3 = 4 raw-database and 8 operand slots.
+// tcgen05 kernel for the fp16 form on the balanced-digit database (block pairs, one launch per 1,024
+// columns): 1 = free-running pairs, 2 = with the wave bound between pairs (cooperative launch) and the
+// moduli in groups of six, 3 = with the wave bound and all moduli in one group.
 #define ICM_CRT_TCGEN05 1
 #define ICM_CRT_TCGEN05_LAST 3
 inline bool crt_tc_variant(int v) { return v >= ICM_CRT_TCGEN05 && v <= ICM_CRT_TCGEN05_LAST; }
@@ -76,21 +72,27 @@ cudaError_t launch_ppmm_crt_tc(const I8Consts &k, const ChunkTab &tab, const voi
 uint32_t device_status(bool clear);
 // Residue planes of the query operand in the CRT forms.
 //  int8: [L][r][N][Kp], K contiguous.
-//  fp16: per (limb, modulus) the columns are grouped in tiles of 256 (N padded with zero columns)
-//  and K in slabs of 16; every (column tile, slab) pair is one contiguous 8 KB block holding the
-//  256 x 16 operand in the tensor cores' K-major layout without swizzle: the core matrices
-//  (8 columns x 8 consecutive k, 16 bytes per column) of k 0-7 for column groups 0..31, then those
-//  of k 8-15.  One bulk copy moves a block into shared memory as it is; blocks of consecutive
-//  slabs of a column tile are adjacent.
+//  fp16: per (limb, modulus) the columns (N padded with zero columns to a multiple of 256) in rounds
+//  of 1,024.  A round of G x 256 columns is split between the two blocks of a pair: columns [0, 128 G)
+//  and [128 G, 256 G).  A block's half is stored by slabs of 16 k: a slab is one contiguous block
+//  of G tiles of 4 KB, a tile holding 128 columns x 16 k in the tensor cores' K-major layout without
+//  swizzle: for each 8 consecutive k the core matrices (8 columns, 16 bytes per column) of the 16
+//  column groups.  So one copy moves the operands of a block and one or more slabs into shared
+//  memory as they are.
 constexpr uint64_t CRT_F16_TN = 256;
 __host__ __device__ inline uint64_t crt_f16_ncols(uint64_t N) { return (N + CRT_F16_TN - 1) / CRT_F16_TN * CRT_F16_TN; }
 inline uint64_t crt_plane_bytes(bool f16, uint32_t n_limbs, uint32_t n_mod, uint64_t N, uint64_t Kp) {
     return f16 ? (uint64_t)n_limbs * n_mod * crt_f16_ncols(N) * Kp * 2 : (uint64_t)n_limbs * n_mod * N * Kp;
 }
-// fp16 element offset of (column j, k) within one (limb, modulus) plane of Kp columns of K
-__host__ __device__ __forceinline__ uint64_t crt_f16_off(uint64_t j, uint64_t k, uint64_t Kp) {
-    return ((j >> 8) * (Kp >> 4) + (k >> 4)) * 4096 + ((((k >> 3) & 1) * 32 + ((j & 255) >> 3)) * 8 + (j & 7)) * 8 +
-           (k & 7);
+// fp16 element offset of (column j, k) within one (limb, modulus) plane of N columns and Kp of K
+// (Kp a multiple of 16)
+__host__ __device__ __forceinline__ uint64_t crt_f16_off(uint64_t j, uint64_t k, uint64_t N, uint64_t Kp) {
+    const uint64_t r0 = j & ~1023ull;                                    // first column of the round
+    const uint64_t left = crt_f16_ncols(N) - r0;
+    const uint32_t G = left < 1024 ? (uint32_t)(left >> 8) : 4u;
+    const uint32_t jj = (uint32_t)(j & 1023), half = jj >= 128 * G ? 1u : 0u, c = jj - half * 128 * G;
+    return r0 * Kp + ((half * (Kp >> 4) + (k >> 4)) * G + (c >> 7)) * 2048 + ((k >> 3) & 1) * 1024 +
+           ((c & 127) >> 3) * 64 + (c & 7) * 8 + (k & 7);
 }
 // small-modulus CRT forms (int8 or fp16 operands): query residue planes, two-phase product.
 // The limbs are processed in groups whose residue bytes stay within CRT_SCRATCH_CAP (at least one

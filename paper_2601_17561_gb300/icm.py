@@ -407,7 +407,7 @@ def icm_autotune(ctx, dbs, q, dev_outs, out_bytes, dev_ws, ws_bytes, stream=None
 
 
 # CRT product kernel variants in the autotuner's order (icm_autotune's ms_per_choice)
-VARIANTS = {128: "mma.sync-128", 256: "mma.sync-256", 1: "tcgen05-r8s4", 2: "tcgen05-r8s4-wave", 3: "tcgen05-r4s8"}
+VARIANTS = {128: "mma.sync-128", 256: "mma.sync-256", 1: "tcgen05-pair", 2: "tcgen05-pair-wave", 3: "tcgen05-pair-wave-allmod"}
 
 
 def icm_ctx_set_variant(ctx, variant: int):
