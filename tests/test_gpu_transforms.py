@@ -41,3 +41,20 @@ def test_encryption_ring_edges(log_n_db, log_n_q, L, Lq, n_db, n_eyes):
     A = O.db_rows(P, W.db_codes, W.db_masks, O.db_layout(n_db, P.ndb, P.rho))
     db = eng.encrypt_db(W.db_codes, W.db_masks)
     assert np.array_equal(_from_digit_form(_u64(db.buf, A.shape), P.q), A)
+
+
+@pytest.mark.parametrize("log_n_db,log_n_q,L,Lq,n_db,n_eyes", SHAPES)
+def test_decryption_ring_edges(log_n_db, log_n_q, L, Lq, n_db, n_eyes):
+    """Decryption (one cluster of L blocks per column, several b-blocks, a partial last one) gives the
+    cleartext inner products exactly, at the full level and after the rescaling."""
+    B.build()
+    prm = dict(log_n_db=log_n_db, log_n_q=log_n_q, n_limbs=L, n_limbs_q=Lq, prime_bits=60,
+               log2_delta=60 if Lq == 2 else 40, seed=9)
+    W = synth.make_workload(n_eyes=n_eyes, n_db=n_db, seed=21)
+    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    db = eng.encrypt_db(W.db_codes, W.db_masks)
+    s = eng.match(db, eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), n_eyes, "u64"))
+    rc, rm = O.rotated_templates(W.q_codes, W.q_masks, eng.rho)
+    want = O.inner_from_counts(*O.hd_counts(rc, rm, O.unpack(W.db_codes), O.unpack(W.db_masks)))
+    assert np.array_equal(eng.decrypt(s).cpu().numpy(), want)
+    assert np.array_equal(eng.decrypt(eng.rescale(s)).cpu().numpy(), want)
