@@ -40,12 +40,6 @@ uint64_t powmod_h128(uint64_t b, uint64_t e, uint64_t q) {
     while (e) { if (e & 1) r = mulmod_h128(r, b, q); b = mulmod_h128(b, b, q); e >>= 1; }
     return r;
 }
-uint64_t shoup_h(uint64_t w, uint64_t q) { return (uint64_t)(((u128)w << 64) / q); }
-uint32_t bitrev(uint32_t x, uint32_t bits) {
-    uint32_t r = 0;
-    for (uint32_t i = 0; i < bits; ++i) r |= ((x >> i) & 1u) << (bits - 1 - i);
-    return r;
-}
 }  // namespace
 
 struct SlotTables {
@@ -53,15 +47,12 @@ struct SlotTables {
     double2 *twist = nullptr;     // [n]   zeta^i
     double2 *tw = nullptr;        // [n/2] omega^k
     int32_t *pos = nullptr;       // [n]   m_j
-    uint64_t *ntt = nullptr;      // [Lq][4][N] psi_rev, psi_rev Shoup, psi^-1 rev, psi^-1 rev Shoup
-    uint64_t ninv[2] = {0, 0}, ninvs[2] = {0, 0};
-    uint64_t q[2] = {0, 0}, rhi[2] = {0, 0}, rlo[2] = {0, 0};
+    uint64_t rhi[2] = {0, 0}, rlo[2] = {0, 0};
     uint64_t q0inv_mod_q1 = 0;    // q_0^-1 mod q_1 (CRT of two limbs)
     ~SlotTables() {
         if (twist) cudaFree(twist);
         if (tw) cudaFree(tw);
         if (pos) cudaFree(pos);
-        if (ntt) cudaFree(ntt);
     }
 };
 
@@ -69,8 +60,8 @@ void free_slot_tables(SlotTables *t) { delete t; }
 
 static std::mutex g_slot_mu;
 
-// Tables of the slot transforms and NTTs for ring degree N_db and the limbs of Q (built once per
-// context, on the context's device).
+// Tables of the slot transforms for ring degree N_db (built once per context, on the context's
+// device).
 static const SlotTables *slot_tables(icm_ctx *c, std::string &why) {
     std::lock_guard<std::mutex> lk(g_slot_mu);
     if (c->slot_tab) return c->slot_tab;
@@ -95,40 +86,14 @@ static const SlotTables *slot_tables(icm_ctx *c, std::string &why) {
         pos[j] = (int32_t)((e - 1) / 4);
         e = e * 5 % (2ull * N);
     }
-    std::vector<uint64_t> ntt((size_t)Lq * 4 * N);
-    uint32_t logN = logn + 1;
-    for (uint32_t l = 0; l < Lq; ++l) {
-        const uint64_t q = c->q[l];
-        if ((q - 1) % (2ull * N)) { delete T; why = "primes must be 1 mod 2 N_db"; return nullptr; }
-        // psi: a primitive 2N-th root of unity, g^((q-1)/2N) for a quadratic non-residue g
-        uint64_t psi = 0;
-        for (uint64_t g = 2; g < 1000 && !psi; ++g)
-            if (powmod_h128(g, (q - 1) / 2, q) == q - 1) psi = powmod_h128(g, (q - 1) / (2ull * N), q);
-        if (!psi || powmod_h128(psi, N, q) != q - 1) { delete T; why = "no primitive 2N-th root"; return nullptr; }
-        const uint64_t ipsi = powmod_h128(psi, q - 2, q);
-        uint64_t *pr = &ntt[((size_t)l * 4 + 0) * N], *prs = &ntt[((size_t)l * 4 + 1) * N];
-        uint64_t *ir = &ntt[((size_t)l * 4 + 2) * N], *irs = &ntt[((size_t)l * 4 + 3) * N];
-        uint64_t pw = 1, ipw = 1;
-        for (uint32_t k = 0; k < N; ++k) {
-            const uint32_t r = bitrev(k, logN);
-            pr[r] = pw; prs[r] = shoup_h(pw, q);
-            ir[r] = ipw; irs[r] = shoup_h(ipw, q);
-            pw = mulmod_h128(pw, psi, q);
-            ipw = mulmod_h128(ipw, ipsi, q);
-        }
-        T->ninv[l] = powmod_h128(N, q - 2, q);
-        T->ninvs[l] = shoup_h(T->ninv[l], q);
-        T->q[l] = q; T->rhi[l] = c->crt.rhi[l]; T->rlo[l] = c->crt.rlo[l];
-    }
+    for (uint32_t l = 0; l < Lq; ++l) { T->rhi[l] = c->crt.rhi[l]; T->rlo[l] = c->crt.rlo[l]; }
     if (Lq == 2) T->q0inv_mod_q1 = powmod_h128(c->q[0] % c->q[1], c->q[1] - 2, c->q[1]);
     cudaError_t err = cudaMalloc(&T->twist, n * sizeof(double2));
     if (err == cudaSuccess) err = cudaMalloc(&T->tw, tw.size() * sizeof(double2));
     if (err == cudaSuccess) err = cudaMalloc(&T->pos, n * sizeof(int32_t));
-    if (err == cudaSuccess) err = cudaMalloc(&T->ntt, ntt.size() * sizeof(uint64_t));
     if (err == cudaSuccess) err = cudaMemcpy(T->twist, twist.data(), n * sizeof(double2), cudaMemcpyHostToDevice);
     if (err == cudaSuccess) err = cudaMemcpy(T->tw, tw.data(), tw.size() * sizeof(double2), cudaMemcpyHostToDevice);
     if (err == cudaSuccess) err = cudaMemcpy(T->pos, pos.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice);
-    if (err == cudaSuccess) err = cudaMemcpy(T->ntt, ntt.data(), ntt.size() * sizeof(uint64_t), cudaMemcpyHostToDevice);
     if (err != cudaSuccess) { delete T; why = cudaGetErrorString(err); return nullptr; }
     c->slot_tab = T;
     return T;
@@ -175,38 +140,6 @@ __device__ __forceinline__ uint64_t mulmod_r128(uint64_t a, uint64_t b, uint64_t
 #pragma unroll 1
     for (int i = 0; i < 5 && r >= q; ++i) r -= q;
     return r;
-}
-
-// Negacyclic NTT of N = 2^logN residues in shared memory (forward: Cooley-Tukey with psi_rev,
-// output in bit-reversed order; inverse: Gentleman-Sande with psi^-1 rev, input in bit-reversed
-// order, scaled by N^-1).  Ends with a barrier.
-__device__ void ntt_fwd(uint64_t *a, uint32_t N, const uint64_t *pr, const uint64_t *prs, uint64_t q) {
-    for (uint32_t m = 1, t = N >> 1; m < N; m <<= 1, t >>= 1) {
-        for (uint32_t b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const uint32_t i = b / t, jj = b & (t - 1);
-            const uint32_t j1 = 2 * i * t + jj, j2 = j1 + t;
-            const uint64_t U = a[j1], V = mulmod_shoup(a[j2], pr[m + i], prs[m + i], q);
-            a[j1] = add_mod(U, V, q);
-            a[j2] = sub_mod(U, V, q);
-        }
-        __syncthreads();
-    }
-}
-__device__ void ntt_inv(uint64_t *a, uint32_t N, const uint64_t *ir, const uint64_t *irs, uint64_t q, uint64_t ninv,
-                        uint64_t ninvs) {
-    for (uint32_t m = N, t = 1; m > 1; m >>= 1, t <<= 1) {
-        const uint32_t h = m >> 1;
-        for (uint32_t b = threadIdx.x; b < N / 2; b += blockDim.x) {
-            const uint32_t i = b / t, jj = b & (t - 1);
-            const uint32_t j1 = 2 * i * t + jj, j2 = j1 + t;
-            const uint64_t U = a[j1], V = a[j2];
-            a[j1] = add_mod(U, V, q);
-            a[j2] = mulmod_shoup(sub_mod(U, V, q), ir[h + i], irs[h + i], q);
-        }
-        __syncthreads();
-    }
-    for (uint32_t j = threadIdx.x; j < N; j += blockDim.x) a[j] = mulmod_shoup(a[j], ninv, ninvs, q);
-    __syncthreads();
 }
 
 __device__ __forceinline__ int tbit(const uint8_t *p, uint64_t b) { return (p[b >> 3] >> (b & 7)) & 1; }
@@ -347,40 +280,42 @@ __global__ void __launch_bounds__(512) k_mu_encode(MuArgs a) {
     }
 }
 
-struct NttTab {
-    const uint64_t *tab;            // [Lq][4][N]
-    uint64_t q[2], ninv[2], ninvs[2], rhi[2], rlo[2];
-};
-
-// Forward NTT of polynomials: poly p of limb l reads src + l src_ls + p src_ps and writes
-// dst + l dst_ls + p dst_ps (N words each).
+// Forward transform of polynomials: poly p of limb l reads src + l src_ls + p src_ps and writes
+// dst + l dst_ls + p dst_ps (N words each, below q).
 struct FwdArgs {
-    NttTab T;
+    icm::NttMod nt[2];
     uint32_t N, Lq, per_limb;
     const uint64_t *src; uint64_t src_ls, src_ps;
     uint64_t *dst; uint64_t dst_ls, dst_ps;
 };
-__global__ void __launch_bounds__(1024) k_ntt_fwd(FwdArgs a) {
+__global__ void __launch_bounds__(512) k_ntt_fwd(const __grid_constant__ FwdArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t total = (uint64_t)a.Lq * a.per_limb;
     for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
         const uint32_t l = (uint32_t)(x / a.per_limb);
         const uint64_t p = x % a.per_limb;
+        const icm::NttMod &T = a.nt[l];
+        const uint64_t q = T.q;
         const uint64_t *s = a.src + l * a.src_ls + p * a.src_ps;
-        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[i] = s[i];
+        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[icm::ntt_pad(i)] = s[i];
         __syncthreads();
-        const uint64_t *tb = a.T.tab + (uint64_t)l * 4 * a.N;
-        ntt_fwd(su, a.N, tb, tb + a.N, a.T.q[l]);
+        icm::ntt_forward(su, 1, 0, a.N, T);
         uint64_t *dd = a.dst + l * a.dst_ls + p * a.dst_ps;
-        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) dd[i] = su[i];
+        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) {
+            uint64_t v = su[icm::ntt_pad(i)];                            // below 4q
+            v = v >= 2 * q ? v - 2 * q : v;
+            dd[i] = v >= q ? v - q : v;
+        }
         __syncthreads();
     }
 }
 
 // Output (limb l, column j, block t, part h): part 0 = a_j mu_{j,t}, part 1 = b_{j,t} mu_{j,t};
-// a_ntt holds NTT(a_j), mu_ntt NTT(mu_{j,t}); b rows are read from the rescaled scores.
+// a_ntt holds NTT(a_j), mu_ntt NTT(mu_{j,t}); b rows are read from the rescaled scores.  The
+// transforms' integer products bound it; with three levels per pass over shared memory (ntt.cuh) the
+// normalisation of 8 eyes x 4,096 templates (N_db = 2^13) takes 717 us, 820 us with one level per pass.
 struct MulArgs {
-    NttTab T;
+    icm::NttMod nt[2];
     uint32_t N, Lq, n_cols, n_blocks;
     uint64_t M;                     // rows of the scores
     const uint64_t *scores;         // [Lq][n_cols][M]
@@ -388,7 +323,7 @@ struct MulArgs {
     const uint64_t *mu_ntt;         // [Lq][n_cols][n_blocks][N]
     uint64_t *out;                  // [Lq][n_cols][n_blocks][2][N]
 };
-__global__ void __launch_bounds__(1024) k_ntt_mul_inv(MulArgs a) {
+__global__ void __launch_bounds__(512) k_ntt_mul_inv(const __grid_constant__ MulArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t per_limb = (uint64_t)a.n_cols * a.n_blocks * 2;
     const uint64_t total = (uint64_t)a.Lq * per_limb;
@@ -398,25 +333,24 @@ __global__ void __launch_bounds__(1024) k_ntt_mul_inv(MulArgs a) {
         const uint32_t h = (uint32_t)(r & 1);
         const uint64_t jt = r >> 1;                                   // j n_blocks + t
         const uint32_t j = (uint32_t)(jt / a.n_blocks), t = (uint32_t)(jt % a.n_blocks);
-        const uint64_t q = a.T.q[l];
-        const uint64_t *tb = a.T.tab + (uint64_t)l * 4 * a.N;
+        const icm::NttMod &T = a.nt[l];
+        const uint64_t q = T.q;
+        const uint64_t *m = a.mu_ntt + (((uint64_t)l * a.n_cols + j) * a.n_blocks + t) * a.N;
         if (h == 0) {
             const uint64_t *s = a.a_ntt + ((uint64_t)l * a.n_cols + j) * a.N;
-            for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[i] = s[i];
-            __syncthreads();
+            for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[icm::ntt_pad(i)] = icm::mul_r128_lazy(s[i], m[i], T);
         } else {
             const uint64_t *s = a.scores + ((uint64_t)l * a.n_cols + j) * a.M + a.N + (uint64_t)t * a.N;
-            for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[i] = s[i];
+            for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) su[icm::ntt_pad(i)] = s[i];
             __syncthreads();
-            ntt_fwd(su, a.N, tb, tb + a.N, q);
+            icm::ntt_forward(su, 1, 0, a.N, T);
+            for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x)
+                su[icm::ntt_pad(i)] = icm::mul_r128_lazy(su[icm::ntt_pad(i)], m[i], T);
         }
-        const uint64_t *m = a.mu_ntt + (((uint64_t)l * a.n_cols + j) * a.n_blocks + t) * a.N;
-        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x)
-            su[i] = mulmod_r128(su[i], m[i], q, a.T.rhi[l], a.T.rlo[l]);
         __syncthreads();
-        ntt_inv(su, a.N, tb + 2 * a.N, tb + 3 * a.N, q, a.T.ninv[l], a.T.ninvs[l]);
+        icm::ntt_inverse(su, 1, 0, a.N, T);
         uint64_t *o = a.out + ((((uint64_t)l * a.n_cols + j) * a.n_blocks + t) * 2 + h) * a.N;
-        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) o[i] = su[i];
+        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) o[i] = mulmod_shoup(su[icm::ntt_pad(i)], T.ninv, T.ninvs, q);
         __syncthreads();
     }
 }
@@ -516,16 +450,6 @@ int sm_count() {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms > 0 ? sms : 1;
-}
-
-NttTab ntt_tab(const SlotTables *T) {
-    NttTab t{};
-    t.tab = T->ntt;
-    for (uint32_t l = 0; l < T->Lq; ++l) {
-        t.q[l] = T->q[l]; t.ninv[l] = T->ninv[l]; t.ninvs[l] = T->ninvs[l];
-        t.rhi[l] = T->rhi[l]; t.rlo[l] = T->rlo[l];
-    }
-    return t;
 }
 
 template <typename K>
@@ -717,34 +641,35 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
         SL_TRY(cudaGetLastError());
     }
     // 3. NTT of every mu (in place) and of every a-part
-    const NttTab NT = ntt_tab(T);
-    const size_t psm = (size_t)N * 8;
+    if (!c->nt.tab_db) return sfail(ICM_EINVAL, "icm_keygen has not run");
+    const size_t psm = (size_t)ntt_words(N) * 8;
     SL_TRY(set_smem(k_ntt_fwd, psm));
     SL_TRY(set_smem(k_ntt_mul_inv, psm));
-    const unsigned per_sm = psm > 110000 ? 1 : (psm > 70000 ? 2 : 4);
-    // one polynomial per block in shared memory: the largest rings fit one block per SM, which
-    // then takes 1,024 threads to hide the latency of the butterflies' 64-bit products
-    const unsigned ntt_threads = psm > 70000 ? 1024 : 512;
+    // one polynomial per block in shared memory, as many blocks per SM as fit
+    const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(4, (size_t)220 * 1024 / psm));
     {
         FwdArgs a{};
-        a.T = NT; a.N = N; a.Lq = Lq; a.per_limb = d3 * nb;
+        for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];
+        a.N = N; a.Lq = Lq; a.per_limb = d3 * nb;
         a.src = mu; a.src_ls = (uint64_t)d3 * nb * N; a.src_ps = N;
         a.dst = mu; a.dst_ls = a.src_ls; a.dst_ps = N;
-        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(a);
+        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * per_sm), 512, psm, st>>>(a);
         SL_TRY(cudaGetLastError());
         FwdArgs b{};
-        b.T = NT; b.N = N; b.Lq = Lq; b.per_limb = d3;
+        for (uint32_t l = 0; l < Lq; ++l) b.nt[l] = c->nt.db[l];
+        b.N = N; b.Lq = Lq; b.per_limb = d3;
         b.src = in->dev; b.src_ls = (uint64_t)d3 * in->lay.M; b.src_ps = in->lay.M;
         b.dst = antt; b.dst_ls = (uint64_t)d3 * N; b.dst_ps = N;
-        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(b);
+        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3, (uint64_t)sms * per_sm), 512, psm, st>>>(b);
         SL_TRY(cudaGetLastError());
     }
     // 4. products and inverse NTTs
     {
         MulArgs a{};
-        a.T = NT; a.N = N; a.Lq = Lq; a.n_cols = d3; a.n_blocks = nb; a.M = in->lay.M;
+        for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];
+        a.N = N; a.Lq = Lq; a.n_cols = d3; a.n_blocks = nb; a.M = in->lay.M;
         a.scores = in->dev; a.a_ntt = antt; a.mu_ntt = mu; a.out = (uint64_t *)dev_out;
-        k_ntt_mul_inv<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb * 2, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(a);
+        k_ntt_mul_inv<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb * 2, (uint64_t)sms * per_sm), 512, psm, st>>>(a);
         SL_TRY(cudaGetLastError());
     }
     return ICM_OK;
