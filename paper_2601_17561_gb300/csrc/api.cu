@@ -776,7 +776,9 @@ icm_status icm_ppmm(icm_form form, const uint64_t *q, uint32_t n_limbs, const ui
             if ((pl || sc) && (!dev_ws || ws_bytes < align256(pl) + sc)) return fail(ICM_ENOMEM, "workspace too small");
             e = launch_crt_planes(f16, k, dev_B, dev_ws, N, K, i8_kpad(K), (cudaStream_t)stream);
             if (e == cudaSuccess)
-                e = launch_ppmm_crt(f16, 256, k, dev_A, false, dev_ws, dev_C, M, N, K, i8_kpad(K),
+                // fp16: the tcgen05 kernel (3 x 3001 x 500 x 8192: 2.05 ms, 12.0 ms on mma.sync) where K and
+                // the operand's alignment allow it
+                e = launch_ppmm_crt(f16, f16 ? 2 : 256, k, dev_A, false, dev_ws, dev_C, M, N, K, i8_kpad(K),
                                     (char *)dev_ws + align256(pl), (cudaStream_t)stream);
             break;
         }

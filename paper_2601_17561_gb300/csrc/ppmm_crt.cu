@@ -471,7 +471,8 @@ cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const C
         }
         return cudaSuccess;
     }
-    if (f16 && crt_tc_variant(bn) && tab.a_digits && crt_tc_supported(K))
+    // canonical operands (icm_ppmm) may have any alignment; the database's is checked when it is built
+    if (f16 && crt_tc_variant(bn) && crt_tc_supported(K) && (tab.a_digits || crt_tc_aligned(tab)))
         return launch_ppmm_crt_tc(k, tab, Bp, N, K, Kp, scratch, bn, st);
     if (bn != 128) bn = 256;
     for (uint64_t n0 = 0; n0 < N; n0 += NCHUNK) {

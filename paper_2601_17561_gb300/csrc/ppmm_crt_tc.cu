@@ -131,6 +131,8 @@ struct TcArgs {
     uint64_t n_tiles;                 // L x row tiles x modulus tiles
     uint32_t *sync;                   // [0]: fetch arrivals (wave bound), [1]: a block gave up; zeroed per launch
     uint64_t wait_ns;                 // bound of every wait
+    uint32_t canonical;               // database words are canonical residues modulo q, not in the storage form
+    uint64_t q[ICM_MAX_LIMBS];
     uint32_t inject_stall;            // test only: the query producers never copy
     uint32_t zero;                    // 0
     TcMod md[ICM_MAX_MODULI];
@@ -506,6 +508,14 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
 #pragma unroll
                     for (int c = 0; c < 4; ++c)
                         z[it][c] = *reinterpret_cast<const ulonglong2 *>(r_s + it * 16 * 128 + (((cj * 4 + c) ^ rsw) << 4));
+                if (p.canonical) {                                       // canonical residues: to the storage form
+                    const uint64_t q = p.q[tc.l];
+#pragma unroll
+                    for (int it = 0; it < ITEMS; ++it)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c)
+                            z[it][c] = make_ulonglong2(to_digit_form(z[it][c].x, q), to_digit_form(z[it][c].y, q));
+                }
 #pragma unroll
                 for (int mu = 0; mu < NM; ++mu) {
                     if (NM > 1 && mu >= (int)tc.nm) break;
@@ -885,9 +895,14 @@ cudaError_t crt_tc_set_attributes() {
     return e;
 }
 
-// The tcgen05 path needs an even K (tensor-map row strides are multiples of 16 bytes); the caller
-// uses the mma.sync kernel otherwise.
+// The tcgen05 path needs an even K and 16-byte aligned chunks (tensor-map base addresses and row
+// strides are multiples of 16 bytes); the caller uses the mma.sync kernel otherwise.
 bool crt_tc_supported(uint64_t K) { return K > 0 && K % 2 == 0; }
+bool crt_tc_aligned(const ChunkTab &tab) {
+    for (uint32_t c = 0; c < tab.n; ++c)
+        if (reinterpret_cast<uintptr_t>(tab.A[c]) % 16) return false;
+    return true;
+}
 
 uint32_t device_status(bool clear) {
     uint32_t v = 0;
@@ -937,6 +952,8 @@ cudaError_t launch_ppmm_crt_tc(const I8Consts &k, const ChunkTab &tab, const voi
     a.n_limbs = k.n_limbs;
     a.wait_ns = k.tc_wait_ns ? k.tc_wait_ns : 2000000000ull;
     a.inject_stall = k.tc_inject_stall;
+    a.canonical = tab.a_digits ? 0u : 1u;
+    for (uint32_t l = 0; l < k.n_limbs; ++l) a.q[l] = k.q[l];
     for (uint32_t i = 0; i < k.n_mod; ++i) {
         const uint32_t m = (uint32_t)k.mod[i];
         uint32_t L = 0x6480;                                             // m <= 255 divides F_0 for some L < 0x6780

@@ -67,6 +67,7 @@ cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const voi
                                uint64_t nch, cudaStream_t st);
 cudaError_t crt_tc_set_attributes();
 bool crt_tc_supported(uint64_t K);
+bool crt_tc_aligned(const ChunkTab &tab);
 cudaError_t launch_ppmm_crt_tc(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
                                void *scratch, int variant, cudaStream_t st);
 uint32_t device_status(bool clear);

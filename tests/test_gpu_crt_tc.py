@@ -43,3 +43,20 @@ def test_column_groups(setup, n_eyes):
     for v in (1, 2, 3):
         for a, b in zip(res[v], res[256]):
             assert np.array_equal(a, b), v
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 2), (127, 31, 34), (129, 257, 1026), (64, 513, 48), (200, 769, 2080), (5, 1025, 96)])
+def test_ppmm_canonical(M, N, K):
+    """Canonical operands through the tcgen05 kernel (even K, 16-byte aligned) and, from an address that is
+    only 8-byte aligned, through mma.sync: both equal to the u64 form."""
+    q = [(1 << 60) - 93, (1 << 50) - 27, (1 << 31) - 1]
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A = torch.stack([torch.randint(0, x, (M, K), generator=g, device="cuda", dtype=torch.int64) for x in q])
+    Bm = torch.stack([torch.randint(0, x, (N, K), generator=g, device="cuda", dtype=torch.int64) for x in q])
+    A[:, 0, :] = torch.tensor(q, device="cuda").view(-1, 1) - 1
+    want = E.ppmm("u64", q, A, Bm)
+    assert torch.equal(E.ppmm("f16_crt", q, A, Bm), want)
+    shifted = torch.empty(A.numel() + 1, dtype=torch.int64, device="cuda")[1:].view(A.shape)
+    shifted.copy_(A)
+    assert shifted.data_ptr() % 16 == 8
+    assert torch.equal(E.ppmm("f16_crt", q, shifted, Bm), want)
