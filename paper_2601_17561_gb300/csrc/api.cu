@@ -416,7 +416,10 @@ icm_status icm_query_prepare(icm_ctx *c, const void *dev_ct, size_t n_eyes, icm_
     if (e == cudaSuccess && form != ICM_FORM_U64) {
         const I8Consts &k = form == ICM_FORM_I8_DIGITS ? c->i8_digits : c->i8_crt;
         int8_t *planes = (int8_t *)dev_op + (size_t)c->p.n_limbs * n_cols * c->K * 8;
-        if (form == ICM_FORM_I8_DIGITS)
+        q->digits = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) && dig_groups(k.n_mod, n_cols, c->K) > 0;
+        if (q->digits)
+            e = launch_dig_planes(k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
+        else if (form == ICM_FORM_I8_DIGITS)
             e = launch_planes(form, k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
         else
             e = launch_crt_planes(form == ICM_FORM_F16_CRT, k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K),
@@ -453,6 +456,7 @@ icm_status icm_match_launches(const icm_ctx *c, const icm_db *db, size_t n_eyes,
     if (form != ICM_FORM_I8_CRT && form != ICM_FORM_F16_CRT) return fail(ICM_EINVAL, "not a match form");
     const uint32_t L = c->p.n_limbs, G = crt_limb_group(L, c->i8_crt.n_mod, N, M);
     const bool tc = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) && crt_tc_supported(c->K);
+    if (tc && dig_groups(c->i8_crt.n_mod, N, c->K)) { *n = 1; return ICM_OK; }
     const uint64_t cols = tc ? 1024 : 512;
     *n = (size_t)((L + G - 1) / G) * ((N + cols - 1) / cols) * 2;
     return ICM_OK;
@@ -483,6 +487,14 @@ icm_status icm_match(icm_ctx *c, const icm_db *db, const icm_query *q, void *dev
         case ICM_FORM_I8_CRT:
         case ICM_FORM_F16_CRT: {
             const void *planes = (const char *)q->dev + (size_t)c->p.n_limbs * q->n_cols * c->K * 8;
+            if (q->digits) {
+                const uint64_t *A = db->dev;
+                uint64_t *C = (uint64_t *)dev_out, M = db->lay.M;
+                ChunkTab tab;
+                make_chunk_tab(&A, &C, &M, 1, tab);
+                e = launch_ppmm_dig(c->i8_crt, tab, planes, q->n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
+                break;
+            }
             e = launch_ppmm_crt(q->form == ICM_FORM_F16_CRT, c->crt_bn, c->i8_crt, db->dev, true, planes,
                                 (uint64_t *)dev_out, db->lay.M, q->n_cols, c->K, i8_kpad(c->K), dev_ws, (cudaStream_t)stream);
             break;

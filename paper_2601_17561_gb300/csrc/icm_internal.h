@@ -107,6 +107,7 @@ struct icm_query {
     const icm_ctx *ctx;
     icm_form form;
     uint32_t n_eyes, n_cols;   // n_cols = d3 = n_eyes * rho
+    bool digits;               // fp16 form: digit planes instead of residue planes
     void *dev;                 // prepared operand
     size_t bytes;
 };

@@ -188,10 +188,15 @@ __device__ __forceinline__ bool mbar_try_rlx(uint32_t bar, uint32_t parity) {
     return ok != 0;
 }
 // Whether the phase of the given parity has completed, without waiting.
+template <bool RLX = false>
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
     uint32_t ok;
-    asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-                 : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    if (RLX)
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.relaxed.cta.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+    else
+        asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+                     : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
 // Shared memory address of this block's `addr` in block `rank` of the cluster.
@@ -210,7 +215,7 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t mapped) {
 // What a bounded wait needs besides its barrier.
 struct WaitCtx {
     volatile int *abort_flag;         // this block's, in shared memory
-    uint32_t *sync;
+    uint32_t *sync;                   // the launch's give-up word follows its wave counter; may be null
     uint64_t wait_ns;
 };
 // A wait ran out: both blocks of the pair stop issuing work.
@@ -221,7 +226,7 @@ __device__ __noinline__ void give_up(const WaitCtx &w) {
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], 1;"
                  :: "r"(map_rank(smem_u32(const_cast<int *>(w.abort_flag)), rank ^ 1u)) : "memory");
     atomicExch(&g_status, (uint32_t)ICM_DEV_TIMEOUT);
-    atomicExch(&w.sync[1], 1u);
+    if (w.sync) atomicExch(&w.sync[1], 1u);
 }
 template <bool RLX>
 __device__ __noinline__ bool mbar_wait_slow(uint32_t bar, uint32_t parity, const WaitCtx &w) {
@@ -820,6 +825,8 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(TMEM_COLS) : "memory");
 }
 
+#include "ppmm_dig_tc.cuh"
+
 // ---------------------------------------------------------------- host side
 
 using EncodeTiled = CUresult (*)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -892,7 +899,82 @@ cudaError_t crt_tc_set_attributes() {
     if (e == cudaSuccess) e = set_attr<Cfg3>();
     if (e == cudaSuccess) e = set_attr<Cfg2>();
     if (e == cudaSuccess) e = set_attr<Cfg1>();
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_dig_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, DG_SMEM);
     return e;
+}
+
+// The digit form takes the fp16 form's product where its planes fit the residue planes' place in the
+// operand (so that buffer sizes do not depend on the choice): up to n_mod / 8 groups of 32 columns,
+// 2 for 60-bit primes, and at most 64 columns.  There one pass of a row tile per group costs 2,048
+// cycles per 16 words and 256 rows, the CRT kernel's conversions 5,500 to 7,400 for any width up to
+// 256 columns (measured: 1 eye x 3,000 codes, 8 limbs: 3.8 ms against 13.1; the product of 2 eyes x 8,192 rows 7.2 against 14.7).
+uint32_t dig_groups(uint32_t n_mod, uint64_t N, uint64_t K) {
+    const uint64_t g = (N + 31) / 32;
+    return N > 0 && g <= 2 && g * 8 <= n_mod && crt_tc_supported(K) ? (uint32_t)g : 0;
+}
+
+cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K, uint64_t Kp,
+                              cudaStream_t st) {
+    if (reinterpret_cast<uintptr_t>(planes) % 16) return cudaErrorInvalidValue;
+    DigPlanesArgs a{};
+    a.op = op; a.planes = reinterpret_cast<unsigned char *>(planes);
+    a.N = N; a.K = K; a.Kp = Kp; a.groups = dig_groups(k.n_mod, N, K);
+    for (uint32_t l = 0; l < k.n_limbs; ++l) {
+        a.q[l] = k.q[l];
+        for (int t = 0; t < 8; ++t) { a.w[l][t] = k.pw8[l][t]; a.ws[l][t] = k.pw8s[l][t]; }
+    }
+    const uint64_t warps = Kp / 8 * a.groups * 8;
+    k_dig_planes<<<dim3((unsigned)std::min<uint64_t>((warps + 7) / 8, 152u * 16u), k.n_limbs), 256, 0, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
+                            cudaStream_t st) {
+    if (tab.row0[tab.n] == 0 || N == 0) return cudaSuccess;
+    if (!crt_tc_aligned(tab) || reinterpret_cast<uintptr_t>(Bp) % 16) return cudaErrorInvalidValue;
+    EncodeTiled enc = encode_fn();
+    if (!enc) return cudaErrorNotSupported;
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    static_assert(sizeof(DigArgs) <= 32000, "kernel parameter space");
+    DigArgs a{};
+    const cuuint32_t estr[3] = {1, 1, 1};
+    for (uint32_t c = 0; c < tab.n; ++c) {
+        const cuuint64_t M = tab.M[c] ? tab.M[c] : 1;
+        const cuuint64_t dims[3] = {K, M, k.n_limbs}, strides[2] = {K * 8, M * K * 8};
+        const cuuint32_t box[3] = {16, DG_ROWS, 1};
+        if (enc(&a.tmA[c], CU_TENSOR_MAP_DATA_TYPE_UINT64, 3, const_cast<uint64_t *>(tab.A[c]), dims, strides, box, estr,
+                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+            return cudaErrorInvalidValue;
+        a.t0[c + 1] = a.t0[c] + (uint32_t)((tab.M[c] + DG_TILE - 1) / DG_TILE);
+    }
+    a.groups = dig_groups(k.n_mod, N, K);
+    const cuuint64_t dims[2] = {256, (cuuint64_t)k.n_limbs * a.groups * 2 * Kp}, strides[1] = {2048};
+    const cuuint32_t box[2] = {256, DG_WORDS};
+    if (enc(&a.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void *>(Bp), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
+        return cudaErrorInvalidValue;
+    a.tab = tab;
+    a.N = N; a.K = K; a.Kp = Kp; a.n_limbs = k.n_limbs;
+    a.n_tiles = (uint64_t)k.n_limbs * a.t0[tab.n] * a.groups;
+    a.wait_ns = k.tc_wait_ns ? k.tc_wait_ns : 2000000000ull;
+    a.inject_stall = k.tc_inject_stall;
+    for (uint32_t l = 0; l < k.n_limbs; ++l) {
+        a.q[l] = k.q[l]; a.r64[l] = k.r64[l]; a.p32[l] = k.pw8[l][4]; a.p32s[l] = k.pw8s[l][4];
+    }
+    cudaLaunchConfig_t cfg = {};
+    cudaLaunchAttribute attr[1];
+    cfg.gridDim = dim3(2 * (unsigned)std::min<uint64_t>(a.n_tiles, (uint64_t)(sms / 2)));
+    cfg.blockDim = dim3(DG_THREADS);
+    cfg.dynamicSmemBytes = DG_SMEM;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_dig_tc, a);
 }
 
 // The tcgen05 path needs an even K and 16-byte aligned chunks (tensor-map base addresses and row

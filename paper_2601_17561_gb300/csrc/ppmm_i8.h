@@ -68,6 +68,13 @@ cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const voi
 cudaError_t crt_tc_set_attributes();
 bool crt_tc_supported(uint64_t K);
 bool crt_tc_aligned(const ChunkTab &tab);
+// Digit form of the fp16 product for few columns (ppmm_dig_tc.cuh): column groups of 32, or 0 where the
+// CRT form is taken; its planes lie where the residue planes would.
+uint32_t dig_groups(uint32_t n_mod, uint64_t N, uint64_t K);
+cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K, uint64_t Kp,
+                              cudaStream_t st);
+cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
+                            cudaStream_t st);
 cudaError_t launch_ppmm_crt_tc(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
                                void *scratch, int variant, cudaStream_t st);
 uint32_t device_status(bool clear);

@@ -45,6 +45,59 @@ def test_column_groups(setup, n_eyes):
             assert np.array_equal(a, b), v
 
 
+@pytest.fixture(scope="module")
+def wide():
+    # 60-bit primes (18 CRT moduli), K = 2^14 + 2^7: an odd number of 16-word slabs over whole stages
+    eng = E.Engine(log_n_db=7, log_n_q=7, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=8,
+                   hamming_weight=64).keygen()
+    W = synth.make_workload(n_eyes=3, n_db=500, seed=33)
+    cuts = [0, 3, 400, 500]
+    dbs = [eng.encrypt_db(W.db_codes[a:b], W.db_masks[a:b], chunk_id=i) for i, (a, b) in enumerate(zip(cuts, cuts[1:]))]
+    return eng, W, dbs
+
+
+def _both(eng, dbs, ct, n_eyes):
+    """Residues of the fp16 form on tcgen05 (digits up to 64 columns) and of the u64 form."""
+    out = []
+    for form in ("f16_crt", "u64"):
+        s = eng.match_batch(dbs, eng.prepare(ct, n_eyes, form))
+        torch.cuda.synchronize()
+        out.append([x.residues() for x in s])
+    C.icm_device_status(True)
+    return out
+
+
+@pytest.mark.parametrize("n_eyes,launches", [(1, 1), (2, 1), (3, 2)])
+def test_few_columns(wide, n_eyes, launches):
+    """31 and 62 columns multiply digits (one and two groups of 32 columns), 93 residues."""
+    eng, W, dbs = wide
+    assert C.icm_match_launches(eng.ctx, dbs[0].handle, n_eyes, C.FORMS["f16_crt"]) == launches
+    ct = eng.encrypt_query(W.q_codes[:n_eyes], W.q_masks[:n_eyes], W.eye_ids[:n_eyes])
+    a, b = _both(eng, dbs, ct, n_eyes)
+    for x, y in zip(a, b):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("sign", [1, -1])
+def test_few_columns_extreme_digits(wide, sign):
+    """Every database word and query coefficient at the value whose seven low digits are -128 (times
+    the sign for the query): the first digits' products are all 2^14, the accumulators' bound."""
+    eng, _, dbs = wide
+    v = -sum(128 * 256 ** t for t in range(7))
+    z = int.from_bytes(bytes([0x80] * 7 + [0]), "little")
+    db = dbs[1]
+    keep = db.buf.clone()
+    try:
+        db.buf.view(torch.int64).fill_(z)
+        ct = torch.full((31 * eng.K,), (sign * v) % eng.primes[0], dtype=torch.int64, device=eng.device).view(torch.uint8)
+        a, b = _both(eng, [db], ct, 1)
+        assert np.array_equal(a[0], b[0])
+        want = [(sign * v * v * eng.K) % q for q in eng.primes]
+        assert all(np.all(a[0][l] == w) for l, w in enumerate(want))
+    finally:
+        db.buf.copy_(keep)
+
+
 @pytest.mark.parametrize("M,N,K", [(1, 1, 2), (127, 31, 34), (129, 257, 1026), (64, 513, 48), (200, 769, 2080), (5, 1025, 96)])
 def test_ppmm_canonical(M, N, K):
     """Canonical operands through the tcgen05 kernel (even K, 16-byte aligned) and, from an address that is
