@@ -21,8 +21,8 @@
 //   issues inside a lane-dependent branch and 40 on a successful barrier probe, beside the
 //   converters' issue slots; copies of 4 to 16 KB took it ~383 cycles each, so one copy per 16-deep
 //   slab and producer cannot feed a 256-cycle slab, while L2 itself delivers 117 B/clk/SM to several
-//   threads.  Here an operand stage is 32 deep (one copy of up to 32 KB per modulus), two raw
-//   producers alternate, and producers and issuer run on warp-uniform values with one elected lane.
+//   threads.  Here an operand stage is 32 deep (one copy of up to 32 KB per modulus), 
+//   and producers and issuer run on warp-uniform values with one elected lane.
 //   The MMA runs at 71 cycles for M 256 N 128 K 16 (64 is the peak; N 256 reaches 128 of 128, but
 //   needs twice the conversions): 570 cycles per 32-deep stage.
 //   Measured (GB300): 32 eyes against N_db + 16,384 rows, 8 limbs: 218 -> 168 ms per pass; 734 cycles
@@ -34,15 +34,15 @@
 //   at 512 columns), moduli in groups of 3 / 9 instead of 6 (+1 / +3 %).
 //
 // Pipeline, the stages decoupled by rings of shared-memory slots with "full" / "empty" mbarriers:
-//  * raw producers (2 warps per block, alternate slabs): one TMA load per 16-deep slab of the 64 x
+//  * raw producer (1 warp per block): one TMA load per 16-deep slab of the 64 x
 //    16 balanced-digit storage words of the block's rows (128-byte swizzle: the 16-byte chunk c of
 //    row r sits at chunk c ^ (r mod 8)) into a ring of RS raw slots;
 //  * converters (8 warps in NCG = 4 groups): the group of slab g (g mod NCG) converts it, each warp
 //    32 rows: 8 consecutive storage words of a row become 8 fp16 residues in registers, then, once
 //    the operand stage is free, 16-byte stores into the MMA's K-major core-matrix layout (no
 //    swizzle);
-//  * query producers (1 warp per modulus of the tile and block): per stage one TMA load of the block's
-//    pre-tiled plane block, signalled on the leader's barrier;
+//  * query producer (1 warp per block): per stage and modulus one TMA load of the block's pre-tiled plane
+//    block, signalled on the leader's barrier;
 //  * MMA issuer (leader block only): per stage one wait, two tcgen05.mma (cta_group::2) per accumulator
 //    and one commit to both blocks.  The leader's "full" barrier of a stage counts the converter
 //    warps of both blocks and the bytes of both blocks' planes;
@@ -85,7 +85,6 @@ constexpr int NCG = 4, WPG = 2, NCV = NCG * WPG;  // converter groups, warps per
 constexpr int ROWS_W = ROWS / WPG, ITEMS = ROWS_W / 16;   // rows of a converter warp, in items of 16
 constexpr int NEP = 8;                            // epilogue warps: two per TMEM lane quarter
 constexpr int EP_COLS = BM / 2;                   // accumulator columns of one epilogue warp
-constexpr int NRAW = 2;                           // raw producers
 constexpr uint64_t LAUNCH_COLS = 1024;            // columns of one launch: the scratch width
 
 // Configuration of a launch: G column groups of 256 x NM moduli per tile, S operand stages of KH slabs,
@@ -99,7 +98,7 @@ struct Cfg {
     static constexpr int Q_STAGE = NM * Q_MOD, R_STAGE = NM * KH * R_BLK;
     static constexpr int OFF_Q = RS * RAW_SLOT, OFF_R = OFF_Q + S * Q_STAGE, BARS = OFF_R + S * R_STAGE;
     static constexpr int SMEM = BARS + 1024 + 1024;   // barriers + slack to align the base to 1024
-    static constexpr int W_EPI = NCV, W_RAW = NCV + NEP, W_QRY = W_RAW + NRAW, W_MMA = W_QRY + NM;
+    static constexpr int W_EPI = NCV, W_RAW = NCV + NEP, W_QRY = W_RAW + 1, W_MMA = W_QRY + 1;
     static constexpr int NTHREADS = (W_MMA + 1) * 32;
     static constexpr uint32_t KST = KS * KH;          // K of a stage
     static constexpr uint32_t FLUSH = FLUSH_K / KST;  // stages between an accumulator's reductions
@@ -109,7 +108,6 @@ struct Cfg {
     static_assert(NACC * BM <= (int)TMEM_COLS, "accumulators");
     static_assert(SMEM <= 227 * 1024, "shared memory budget");
     static_assert(RS % NCG == 0 && (KH * S) % NCG == 0, "a slot always belongs to one converter group");
-    static_assert(RS % NRAW == 0, "a raw slot always belongs to one producer");
 };
 
 struct TcMod {
@@ -353,6 +351,7 @@ struct ResMod {
     int wlo, whi, f0;
     uint32_t hneg2;
     uint64_t inv, k1, nm;
+    __device__ __forceinline__ ResMod() {}
     __device__ __forceinline__ explicit ResMod(const TcMod &t)
         : wlo(t.wlo), whi(t.whi), f0((int)t.f0), hneg2(t.hneg2), inv(dup2(t.inv_m)), k1(dup2(t.k1)), nm(dup2(-t.m)) {}
 };
@@ -481,7 +480,7 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
     const uint32_t nk = nst * KH;                                  // slabs of a tile
     const uint64_t Mall = p.tab.row0[p.tab.n];
     const uint32_t t_first = blockIdx.x >> 1, t_step = gridDim.x >> 1;   // persistent tile sequence of the pair
-    constexpr uint32_t FETCHERS = NRAW + NM;
+    constexpr uint32_t FETCHERS = 2;
 
     if (warp < NCV) {
         // ------------------------------------------------------------------ converter warps
@@ -504,6 +503,9 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
         for (uint64_t tile = t_first; alive && tile < p.n_tiles; tile += t_step) {
             const TileCoord tc = tile_coord<NM>(p, tile);
             g_end += nk;                                                 // the groups' turns continue across tiles
+            ResMod mds[NM];                                              // constants of the tile's moduli
+#pragma unroll
+            for (int mu = 0; mu < NM; ++mu) mds[mu] = ResMod(p.md[min(tc.mi0 + mu, p.n_mod - 1)]);
             for (; g < g_end; g += NCG) {
                 if (!mbar_wait(b_rawfull + rs * 8, rpar, wc)) { alive = false; break; }
                 const unsigned char *r_s = sW + rs * RAW_SLOT + lrow0 * 128;
@@ -524,7 +526,7 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
 #pragma unroll
                 for (int mu = 0; mu < NM; ++mu) {
                     if (NM > 1 && mu >= (int)tc.nm) break;
-                    const ResMod md(p.md[tc.mi0 + mu]);
+                    const ResMod &md = mds[mu];
                     uint32_t w[ITEMS][4];
 #pragma unroll
                     for (int it = 0; it < ITEMS; ++it)
@@ -646,31 +648,27 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
             }
         }
     } else if (warp < C::W_QRY) {
-        // ------------------------------------------------------------------ raw database producers
+        // ------------------------------------------------------------------ raw database producer
         // The producers' and the issuer's loops run in whole warps on uniform values, with one elected
         // lane for the copies and MMAs: a copy issued inside a lane-dependent branch costs 51 cycles,
         // an elected one 17.
-        // slabs g with g mod NRAW = part of the pair's whole sequence
         const bool el = elect_one();
-        const uint32_t part = (uint32_t)(warp - C::W_RAW);
-        uint64_t g = part, g0 = 0;                                        // next slab, first slab of the tile
-        uint32_t rs = part, rpar = 0, w = 0;                              // slot, parity of its phase
-        for (uint64_t tile = t_first; tile < p.n_tiles; tile += t_step, ++w, g0 += nk) {
+        uint64_t g = 0;                                                   // slabs issued
+        uint32_t rs = 0, rpar = 0, w = 0;                                 // slot, parity of its phase
+        for (uint64_t tile = t_first; tile < p.n_tiles; tile += t_step, ++w) {
             const TileCoord tc = tile_coord<NM>(p, tile);
             if (SYNC && w && !wave_wait(FETCHERS * gridDim.x * w, wc)) break;
             const int row = (int)(tc.m0 + rank * ROWS);
             const CUtensorMap *map = &p.tmA[tc.c];
             bool alive = true;
-            for (; g < g0 + nk; g += NRAW) {
+            for (uint32_t kt = 0; kt < nk; ++kt, ++g) {
                 if (!mbar_wait(b_rawempty + rs * 8, rpar ^ 1, wc)) { alive = false; break; }
                 if (el) {
                     mbar_expect_tx(b_rawfull + rs * 8, RAW_SLOT);
-                    tma_load_3d(smem_u32(sW) + rs * RAW_SLOT, map, (int)((uint32_t)(g - g0) * KS), row, (int)tc.l,
-                                b_rawfull + rs * 8);
+                    tma_load_3d(smem_u32(sW) + rs * RAW_SLOT, map, (int)(kt * KS), row, (int)tc.l, b_rawfull + rs * 8);
                 }
                 __syncwarp();
-                rs += NRAW;
-                if (rs >= (uint32_t)RS) { rs -= RS; rpar ^= 1; }
+                if (++rs == (uint32_t)RS) { rs = 0; rpar ^= 1; }
             }
             if (!alive) break;
             if (SYNC && el) atomicAdd(&p.sync[0], 1u);
@@ -678,12 +676,11 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
         }
         // every load issued by this warp has landed before the block exits
         const uint64_t deadline = gtime() + p.wait_ns;
-        for (uint64_t i = (g >= (uint64_t)(RS + part) ? g - RS : part); i < g; i += NRAW)
+        for (uint64_t i = g > (uint64_t)RS ? g - RS : 0; i < g; ++i)
             mbar_wait_until(&bars->rawfull[i % RS], (uint32_t)((i / RS) & 1), deadline);
     } else if (warp < C::W_MMA) {
-        // ------------------------------------------------------------------ query plane producers
+        // ------------------------------------------------------------------ query plane producer
         const bool el = elect_one();
-        const uint32_t mu = (uint32_t)(warp - C::W_QRY);                 // modulus of the tile
         const uint32_t full0 = map_rank(b_full, 0);
         uint64_t n = 0, n0 = 0;                                          // next stage, first stage of the tile
         uint32_t s = 0, spar = 0, w = 0;
@@ -691,19 +688,22 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
             const TileCoord tc = tile_coord<NM>(p, tile);
             if (SYNC && w && !wave_wait(FETCHERS * gridDim.x * w, wc)) break;
             // a slab of this block is 2 G rows of 2 KB; the blocks' halves of a round are p.slabs apart
-            // (a tile short of moduli repeats its last one: every producer takes part in every stage,
-            // so that none falls a barrier phase behind)
-            const uint32_t row0 = (uint32_t)(((uint64_t)tc.l * p.n_mod + tc.mi0 + min(mu, tc.nm - 1)) * p.q_plane_rows +
-                                             p.q_row0 + (uint64_t)rank * p.slabs * (2 * G));
+            // (a tile short of moduli repeats its last one, so that the bytes of a stage are always the same)
+            const uint32_t row0 = (uint32_t)(((uint64_t)tc.l * p.n_mod + tc.mi0) * p.q_plane_rows + p.q_row0 +
+                                             (uint64_t)rank * p.slabs * (2 * G));
+            const uint32_t plane_rows = (uint32_t)p.q_plane_rows;
             bool alive = true;
             for (; n < n0 + nst; ++n) {
                 // the stage is free once every accumulator's MMAs that read it have completed
                 if (!mbar_wait(b_empty + s * 8, spar ^ 1, wc)) { alive = false; break; }
                 if (el) {
                     // the leader announces the bytes of both blocks and all moduli
-                    if (rank == 0 && mu == 0) mbar_expect_tx(b_full + s * 8, 2 * C::Q_STAGE);
-                    tma_load_2d_pair(smem_u32(sQ) + s * C::Q_STAGE + mu * C::Q_MOD, &p.tmQ, 0,
-                                     (int)(row0 + (uint32_t)(n - n0) * (2 * G * KH)), full0 + s * 8);
+                    if (rank == 0) mbar_expect_tx(b_full + s * 8, 2 * C::Q_STAGE);
+#pragma unroll
+                    for (int mu = 0; mu < NM; ++mu)
+                        tma_load_2d_pair(smem_u32(sQ) + s * C::Q_STAGE + mu * C::Q_MOD, &p.tmQ, 0,
+                                         (int)(row0 + min((uint32_t)mu, tc.nm - 1) * plane_rows + (uint32_t)(n - n0) * (2 * G * KH)),
+                                         full0 + s * 8);
                 }
                 __syncwarp();
                 if (++s == (uint32_t)S) { s = 0; spar ^= 1; }
