@@ -47,12 +47,22 @@ struct DbMsgArgs {
 
 // Pass 1: the message residues Q' * W[r][k] of every stored b-row, for the limbs of Q (they are zero
 // modulo the limbs of Q', which pass 2 does not read).  The message
-// row is the masked bit-vector c' of template r (coefficient encoding) or, for a slot-encoded
+// row is the masked bit-vector c' of template r (coefficient encoding, BITS) or, for a slot-encoded
 // chunk, the given row of rounded slot-encoding coefficients.
-__global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
-    extern __shared__ unsigned char smem[];
-    int32_t *cp = reinterpret_cast<int32_t *>(smem);                        // [d2]
-    int32_t *spos = cp + ((a.d2 + 3) & ~3u);                                // [nqblk*h]
+//
+// (M_db S_q)[r][j] = sum over the query secrets' non-zeros (position p, sign s) of s e[j + p], e = c'
+// followed by -c' (the negacyclic wrap): h d2 / N_q additions per entry.  With c' in {-1, 0, 1} four
+// entries are added at once as bytes 1 + s c' of a word: the row is kept as 1 + c', 1 - c', 1 + c' (a
+// negative sign starts N_q later), unaligned words come from two aligned ones by a funnel shift, and the
+// bytes are widened every 127 terms.  Shared-memory reads bound it (two words per four additions):
+// 1,030 rows, N_q = 2^13: 0.6 ms, 3.8 ms with one addition at a time.
+template <bool BITS>
+__global__ void __launch_bounds__(512) k_db_messages(const __grid_constant__ DbMsgArgs a) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    // BITS: [nqblk][3 N_q + 4] bytes, else [d2] words; then the supports (BITS: start offsets)
+    const uint32_t stride = 3 * a.Nq + 4;
+    int32_t *cp = reinterpret_cast<int32_t *>(smem);
+    int32_t *spos = reinterpret_cast<int32_t *>(smem + (BITS ? (size_t)a.nqblk * stride : (size_t)((a.d2 + 3) & ~3u) * 4));
     int8_t *ssgn = reinterpret_cast<int8_t *>(spos + a.nqblk * a.h);
 
     const uint64_t bidx = blockIdx.x;
@@ -62,39 +72,7 @@ __global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
     const uint64_t r = (uint64_t)t * a.lay.N + i;
     const bool real = r < a.lay.n_real;
     const uint32_t tb = a.code_bits / 8;
-    for (uint32_t k = threadIdx.x; k < a.d2; k += blockDim.x) {
-        int v = 0;
-        if (real && a.wmsg) {
-            v = a.wmsg[r * a.d2 + k];
-        } else if (real && k < a.code_bits) {
-            const int c = template_bit(a.codes + r * tb, k), m = template_bit(a.masks + r * tb, k);
-            v = m - 2 * (c & m);
-        }
-        cp[k] = v;
-    }
-    for (uint32_t x = threadIdx.x; x < a.nqblk * a.h; x += blockDim.x) { spos[x] = a.sq_pos[x]; ssgn[x] = a.sq_sgn[x]; }
-    __syncthreads();
-
-    for (uint32_t k = threadIdx.x; k < a.K; k += blockDim.x) {
-        int32_t W = 0;
-        if (real) {
-            if (k < a.d2) {
-                W = cp[k];
-            } else {
-                // (M_db S_q)[r][j] = sum_t sum_{k'} c'[t Nq + k'] Neg(s_{q,t})[k'][j]; only k' = (j + p) mod Nq
-                // with s_{q,t}[p] != 0 contribute, with sign -1 when j + p wraps past Nq.
-                const uint32_t j = k - a.d2;
-                for (uint32_t tt = 0; tt < a.nqblk; ++tt) {
-                    const int32_t *crow = cp + tt * a.Nq;
-                    for (uint32_t c = 0; c < a.h; ++c) {
-                        const uint32_t p = (uint32_t)spos[tt * a.h + c];
-                        const int s = ssgn[tt * a.h + c];
-                        const uint32_t jp = j + p;
-                        W += (jp < a.Nq) ? s * crow[jp] : -s * crow[jp - a.Nq];
-                    }
-                }
-            }
-        }
+    auto put = [&](uint32_t k, int32_t W) {
         for (uint32_t l = 0; l < a.Lq; ++l) {
             uint64_t v = 0;
             if (W != 0) {
@@ -103,6 +81,82 @@ __global__ void __launch_bounds__(512) k_db_messages(DbMsgArgs a) {
             }
             a.db[((size_t)l * a.lay.M + pos) * a.K + k] = v;
         }
+    };
+    for (uint32_t k = threadIdx.x; k < a.d2; k += blockDim.x) {
+        int v = 0;
+        if (real && !BITS && a.wmsg) {
+            v = a.wmsg[r * a.d2 + k];
+        } else if (real && k < a.code_bits) {
+            const int c = template_bit(a.codes + r * tb, k), m = template_bit(a.masks + r * tb, k);
+            v = m - 2 * (c & m);
+        }
+        if (!BITS) {
+            cp[k] = v;
+        } else {
+            unsigned char *e = smem + (size_t)(k / a.Nq) * stride + k % a.Nq;
+            e[0] = (unsigned char)(1 + v);
+            e[a.Nq] = (unsigned char)(1 - v);
+            e[2 * a.Nq] = (unsigned char)(1 + v);
+        }
+        put(k, v);
+    }
+    for (uint32_t x = threadIdx.x; x < a.nqblk * a.h; x += blockDim.x) {
+        const int8_t g = a.sq_sgn[x];
+        spos[x] = a.sq_pos[x] + (BITS && g < 0 ? (int32_t)a.Nq : 0);
+        if (!BITS) ssgn[x] = g;
+    }
+    if (BITS)
+        for (uint32_t x = threadIdx.x; x < a.nqblk * 4; x += blockDim.x) smem[(size_t)(x >> 2) * stride + 3 * a.Nq + (x & 3)] = 0;
+    __syncthreads();
+    if (!real) {
+        for (uint32_t k = a.d2 + threadIdx.x; k < a.K; k += blockDim.x) put(k, 0);
+        return;
+    }
+    if (BITS) {
+        const uint32_t nw = a.Nq / 4, terms = a.nqblk * a.h;
+        constexpr int V = 4;                                             // words (of four entries) per thread
+        for (uint32_t w0 = threadIdx.x; w0 < nw; w0 += blockDim.x * V) {
+            uint32_t lo[V] = {}, hi[V] = {};                             // 16-bit sums of the even and odd entries
+            for (uint32_t tt = 0; tt < a.nqblk; ++tt) {
+                const uint32_t *e = reinterpret_cast<const uint32_t *>(smem + (size_t)tt * stride);
+                for (uint32_t c0 = 0; c0 < a.h; c0 += 127) {
+                    const uint32_t c1 = min(c0 + 127, a.h);
+                    uint32_t acc[V] = {};
+                    for (uint32_t c = c0; c < c1; ++c) {
+                        const uint32_t o = (uint32_t)spos[tt * a.h + c], sh = 8 * (o & 3);
+                        const uint32_t *p = e + w0 + (o >> 2);
+#pragma unroll
+                        for (int x = 0; x < V; ++x)
+                            if (w0 + x * blockDim.x < nw)
+                                acc[x] += __funnelshift_r(p[x * blockDim.x], p[x * blockDim.x + 1], sh);
+                    }
+#pragma unroll
+                    for (int x = 0; x < V; ++x) { lo[x] += acc[x] & 0x00FF00FFu; hi[x] += (acc[x] >> 8) & 0x00FF00FFu; }
+                }
+            }
+#pragma unroll
+            for (int x = 0; x < V; ++x) {
+                const uint32_t j = 4 * (w0 + x * blockDim.x);
+                if (j >= a.Nq) continue;
+                put(a.d2 + j, (int32_t)(lo[x] & 0xFFFF) - (int32_t)terms);
+                put(a.d2 + j + 1, (int32_t)(hi[x] & 0xFFFF) - (int32_t)terms);
+                put(a.d2 + j + 2, (int32_t)(lo[x] >> 16) - (int32_t)terms);
+                put(a.d2 + j + 3, (int32_t)(hi[x] >> 16) - (int32_t)terms);
+            }
+        }
+    } else for (uint32_t j = threadIdx.x; j < a.Nq; j += blockDim.x) {
+        // only k' = (j + p) mod Nq with s_{q,t}[p] != 0 contribute, with sign -1 when j + p wraps past Nq
+        int32_t W = 0;
+        for (uint32_t tt = 0; tt < a.nqblk; ++tt) {
+            const int32_t *crow = cp + tt * a.Nq;
+            for (uint32_t c = 0; c < a.h; ++c) {
+                const uint32_t p = (uint32_t)spos[tt * a.h + c];
+                const int s = ssgn[tt * a.h + c];
+                const uint32_t jp = j + p;
+                W += (jp < a.Nq) ? s * crow[jp] : -s * crow[jp - a.Nq];
+            }
+        }
+        put(a.d2 + j, W);
     }
 }
 
@@ -129,7 +183,7 @@ constexpr int NT_MUL = 512;
 // but a transform costs about 7 Shoup products per coefficient.  Columns are taken four at a time
 // where 2^14 words hold them, so that a row's words fill a 32-byte sector and the columns share
 // their twiddles.  1,000 templates at N_db = 2^12, four primes (4.0 GB): 69.5 ms with the
-// additions, 15.3 ms now.
+// additions, 12.1 ms now (11.4 of them here).
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant__ DbEncArgs a) {
     extern __shared__ uint64_t su[];                                     // [2^logc][stride]
@@ -327,11 +381,16 @@ cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uin
     a.db = d_db;
     const uint64_t nb = lay.M - lay.N;
     if (nb == 0) return cudaSuccess;
-    const size_t smem = (size_t)((a.d2 + 3) & ~3u) * 4 + (size_t)a.nqblk * a.h * 5;
-    cudaError_t e = cudaFuncSetAttribute(k_db_messages, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    k_db_messages<<<(unsigned)nb, 512, smem, st>>>(a);
-    return cudaGetLastError();
+    // 16-bit sums of bytes below 3 hold 32,767 terms
+    const bool bits = !d_wmsg && (uint64_t)a.nqblk * a.h < 32768;
+    const size_t smem = (bits ? (size_t)a.nqblk * (3 * a.Nq + 4) : (size_t)((a.d2 + 3) & ~3u) * 4) + (size_t)a.nqblk * a.h * 5;
+    auto run = [&](auto kern) {
+        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+        kern<<<(unsigned)nb, 512, smem, st>>>(a);
+        return cudaGetLastError();
+    };
+    return bits ? run(k_db_messages<true>) : run(k_db_messages<false>);
 }
 
 // Columns per block of the secret-product kernels: as many as 2^14 words hold, at most `want`.
