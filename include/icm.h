@@ -189,9 +189,9 @@ icm_status icm_match_workspace_bytes(const icm_ctx *ctx, const icm_db *db, size_
 /* Kernel launches that icm_match enqueues for n_eyes eyes in `form` on this chunk with the
  * context's current variant: 1 for the u64 and digit forms; for the CRT forms a product launch
  * and a recombination launch per column round (1,024 columns on the tcgen05 kernel, 512 on
- * mma.sync) and per group of limbs (the groups keep the residue scratch within 6 GiB); 1 for the
- * fp16 form on tcgen05 with up to 64 columns (32 where the moduli are fewer than 16), which
- * multiplies digits instead of residues. */
+ * mma.sync) and per group of limbs (the groups keep the residue scratch within 6 GiB); in the
+ * fp16 form on tcgen05 one more launch where the last columns (up to 64 past a multiple of 256) are
+ * multiplied as digits instead of residues, and only that one if there are no others. */
 icm_status icm_match_launches(const icm_ctx *ctx, const icm_db *db, size_t n_eyes, icm_form form, size_t *n);
 
 /* CCMM (Section 2.3): C = [A1 A2; B1 B2] * [B_q; A_q] per limb, i.e. the four plaintext modular

@@ -416,16 +416,24 @@ icm_status icm_query_prepare(icm_ctx *c, const void *dev_ct, size_t n_eyes, icm_
     if (e == cudaSuccess && form != ICM_FORM_U64) {
         const I8Consts &k = form == ICM_FORM_I8_DIGITS ? c->i8_digits : c->i8_crt;
         int8_t *planes = (int8_t *)dev_op + (size_t)c->p.n_limbs * n_cols * c->K * 8;
-        q->digits = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) && dig_groups(k.n_mod, n_cols, c->K) > 0;
-        if (q->digits)
-            e = launch_dig_planes(k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
+        const uint32_t n_dig = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) ? dig_cols(k.n_mod, n_cols, c->K) : 0;
+        q->n_crt = n_cols - n_dig;
+        if (n_dig) {
+            const uint64_t Kp = i8_kpad(c->K);
+            char *dig = (char *)planes + crt_plane_bytes(true, c->p.n_limbs, k.n_mod, q->n_crt, Kp);
+            e = launch_crt_planes(true, k, (const uint64_t *)dev_op, n_cols, planes, q->n_crt, c->K, Kp, (cudaStream_t)stream);
+            if (e == cudaSuccess)
+                e = launch_dig_planes(k, (const uint64_t *)dev_op + (size_t)q->n_crt * c->K, n_cols, dig, n_dig, c->K, Kp,
+                                      (cudaStream_t)stream);
+        }
         else if (form == ICM_FORM_I8_DIGITS)
             e = launch_planes(form, k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
         else
-            e = launch_crt_planes(form == ICM_FORM_F16_CRT, k, (const uint64_t *)dev_op, planes, n_cols, c->K, i8_kpad(c->K),
+            e = launch_crt_planes(form == ICM_FORM_F16_CRT, k, (const uint64_t *)dev_op, n_cols, planes, n_cols, c->K, i8_kpad(c->K),
                                   (cudaStream_t)stream);
     }
     if (e != cudaSuccess) { delete q; return fail(ICM_ECUDA, std::string("query prepare: ") + cudaGetErrorString(e)); }
+    if (form != ICM_FORM_F16_CRT) q->n_crt = n_cols;
     q->ctx = c; q->form = form; q->n_eyes = (uint32_t)n_eyes; q->n_cols = n_cols; q->dev = dev_op; q->bytes = bytes;
     *out = q;
     return ICM_OK;
@@ -456,11 +464,29 @@ icm_status icm_match_launches(const icm_ctx *c, const icm_db *db, size_t n_eyes,
     if (form != ICM_FORM_I8_CRT && form != ICM_FORM_F16_CRT) return fail(ICM_EINVAL, "not a match form");
     const uint32_t L = c->p.n_limbs, G = crt_limb_group(L, c->i8_crt.n_mod, N, M);
     const bool tc = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) && crt_tc_supported(c->K);
-    if (tc && dig_groups(c->i8_crt.n_mod, N, c->K)) { *n = 1; return ICM_OK; }
-    const uint64_t cols = tc ? 1024 : 512;
-    *n = (size_t)((L + G - 1) / G) * ((N + cols - 1) / cols) * 2;
+    const uint64_t cols = tc ? 1024 : 512, n_dig = tc ? dig_cols(c->i8_crt.n_mod, N, c->K) : 0;
+    *n = (size_t)((L + G - 1) / G) * ((N - n_dig + cols - 1) / cols) * 2 + (n_dig ? 1 : 0);
     return ICM_OK;
 }
+
+}  // extern "C"
+
+namespace icm {
+// CRT forms of one prepared query batch: the columns with residue planes, then those with digit planes.
+cudaError_t launch_ppmm_cols(const icm_query *q, int bn, const I8Consts &k, ChunkTab &tab, const void *planes, uint64_t K,
+                             void *scratch, cudaStream_t st) {
+    const bool f16 = q->form == ICM_FORM_F16_CRT;
+    const uint64_t Kp = i8_kpad(K), n_dig = q->n_cols - q->n_crt;
+    tab.n_out = q->n_cols;
+    cudaError_t e = launch_ppmm_crt_grouped(f16, bn, k, tab, planes, q->n_crt, K, Kp, scratch, st);
+    if (e == cudaSuccess && n_dig)
+        e = launch_ppmm_dig(k, tab, (const char *)planes + crt_plane_bytes(true, k.n_limbs, k.n_mod, q->n_crt, Kp), q->n_crt,
+                            n_dig, K, Kp, st);
+    return e;
+}
+}  // namespace icm
+
+extern "C" {
 
 icm_status icm_match(icm_ctx *c, const icm_db *db, const icm_query *q, void *dev_out, size_t bytes, void *dev_ws,
                      size_t ws_bytes, void *stream, icm_scores **out) {
@@ -487,16 +513,11 @@ icm_status icm_match(icm_ctx *c, const icm_db *db, const icm_query *q, void *dev
         case ICM_FORM_I8_CRT:
         case ICM_FORM_F16_CRT: {
             const void *planes = (const char *)q->dev + (size_t)c->p.n_limbs * q->n_cols * c->K * 8;
-            if (q->digits) {
-                const uint64_t *A = db->dev;
-                uint64_t *C = (uint64_t *)dev_out, M = db->lay.M;
-                ChunkTab tab;
-                make_chunk_tab(&A, &C, &M, 1, tab);
-                e = launch_ppmm_dig(c->i8_crt, tab, planes, q->n_cols, c->K, i8_kpad(c->K), (cudaStream_t)stream);
-                break;
-            }
-            e = launch_ppmm_crt(q->form == ICM_FORM_F16_CRT, c->crt_bn, c->i8_crt, db->dev, true, planes,
-                                (uint64_t *)dev_out, db->lay.M, q->n_cols, c->K, i8_kpad(c->K), dev_ws, (cudaStream_t)stream);
+            const uint64_t *A = db->dev;
+            uint64_t *C = (uint64_t *)dev_out, M = db->lay.M;
+            ChunkTab tab;
+            make_chunk_tab(&A, &C, &M, 1, tab);
+            e = launch_ppmm_cols(q, c->crt_bn, c->i8_crt, tab, planes, c->K, dev_ws, (cudaStream_t)stream);
             break;
         }
         default: delete sc; return fail(ICM_EUNSUPPORTED, "form not built");
@@ -786,7 +807,7 @@ icm_status icm_ppmm(icm_form form, const uint64_t *q, uint32_t n_limbs, const ui
             const size_t pl = crt_plane_bytes(f16, n_limbs, k.n_mod, N, i8_kpad(K));
             const size_t sc = crt_scratch_bytes(n_limbs, k.n_mod, N, M);
             if ((pl || sc) && (!dev_ws || ws_bytes < align256(pl) + sc)) return fail(ICM_ENOMEM, "workspace too small");
-            e = launch_crt_planes(f16, k, dev_B, dev_ws, N, K, i8_kpad(K), (cudaStream_t)stream);
+            e = launch_crt_planes(f16, k, dev_B, N, dev_ws, N, K, i8_kpad(K), (cudaStream_t)stream);
             if (e == cudaSuccess)
                 // fp16: the tcgen05 kernel (3 x 3001 x 500 x 8192: 2.05 ms, 12.0 ms on mma.sync) where K and
                 // the operand's alignment allow it

@@ -50,11 +50,7 @@ icm_status enqueue_batch(icm_ctx *c, const icm_db *const *dbs, size_t n, const i
         if (!make_chunk_tab(A.data(), C.data(), M.data(), (uint32_t)n, tab)) return api_fail(ICM_EINVAL, "1..16 chunks");
         tab.a_digits = 1;
         const void *planes = (const char *)q->dev + (size_t)c->p.n_limbs * q->n_cols * c->K * 8;
-        if (q->digits)
-            e = launch_ppmm_dig(c->i8_crt, tab, planes, q->n_cols, c->K, i8_kpad(c->K), st);
-        else
-            e = launch_ppmm_crt_grouped(q->form == ICM_FORM_F16_CRT, bn, c->i8_crt, tab, planes, q->n_cols,
-                                        c->K, i8_kpad(c->K), dev_ws, st);
+        e = launch_ppmm_cols(q, bn, c->i8_crt, tab, planes, c->K, dev_ws, st);
     } else {
         for (size_t i = 0; i < n && e == cudaSuccess; ++i) {
             if (q->form == ICM_FORM_U64)

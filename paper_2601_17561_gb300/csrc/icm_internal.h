@@ -107,7 +107,7 @@ struct icm_query {
     const icm_ctx *ctx;
     icm_form form;
     uint32_t n_eyes, n_cols;   // n_cols = d3 = n_eyes * rho
-    bool digits;               // fp16 form: digit planes instead of residue planes
+    uint32_t n_crt;            // fp16 form: columns with residue planes; digit planes for the others follow
     void *dev;                 // prepared operand
     size_t bytes;
 };
@@ -152,6 +152,8 @@ cudaError_t launch_rescale(const icm_ctx *c, const uint64_t *d_in, uint64_t n, u
 
 cudaError_t build_ntt(icm_ctx *c, std::string &why);
 uint64_t pow_mod(uint64_t b, uint64_t e, uint64_t q);
+cudaError_t launch_ppmm_cols(const icm_query *q, int bn, const I8Consts &k, ChunkTab &tab, const void *planes, uint64_t K,
+                             void *scratch, cudaStream_t st);
 LimbTable make_limb_table(const std::vector<uint64_t> &q);
 uint64_t shoup_of(uint64_t w, uint64_t q);
 

@@ -264,9 +264,9 @@ __global__ void __launch_bounds__(NT, 1) k_crt_p1(P1Args p) {
 }
 
 struct P2Args {
-    icm::ChunkTab tab;       // outputs C_c [L][N][M_c]
+    icm::ChunkTab tab;       // outputs C_c [L][n_out][M_c]
     const uint8_t *R;        // [L][r][nch][sum M_c]
-    uint64_t N, n0, nch;
+    uint64_t n_out, n0, nch;
     icm::I8Consts k;
 };
 
@@ -316,12 +316,12 @@ __global__ void __launch_bounds__(256) k_crt_combine(P2Args p) {
         const uint64_t row = grow - p.tab.row0[c], M = p.tab.M[c];
         const uint64_t S = add_mod(reduce64(Alo[e], q, r64), mulmod_shoup(reduce64(Ahi[e], q, r64), p32, p32s, q), q);
         const uint64_t kappa = (T[e] + (1u << 18)) >> 19;
-        p.tab.C[c][((size_t)l * p.N + p.n0 + col) * M + row] = sub_mod(S, mulmod_shoup(kappa, p.k.Mq[l], p.k.Mqs[l], q), q);
+        p.tab.C[c][((size_t)l * p.n_out + p.n0 + col) * M + row] = sub_mod(S, mulmod_shoup(kappa, p.k.Mq[l], p.k.Mqs[l], q), q);
     }
 }
 
 // int8 residue planes of the query operand: [L][r][N][Kp], zero padded.
-__global__ void __launch_bounds__(256) k_crt_planes_i8(const uint64_t *op, int8_t *planes, uint64_t N, uint64_t K,
+__global__ void __launch_bounds__(256) k_crt_planes_i8(const uint64_t *op, uint64_t n_op, int8_t *planes, uint64_t N, uint64_t K,
                                                        uint64_t Kp, icm::I8Consts k) {
     const uint32_t l = blockIdx.y;
     const uint32_t r = k.n_mod;
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(256) k_crt_planes_i8(const uint64_t *op, int8_
     const uint64_t total = N * Kp;
     for (uint64_t idx = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (uint64_t)gridDim.x * blockDim.x) {
         const uint64_t j = idx / Kp, kk = idx % Kp;
-        const uint64_t v = kk < K ? op[((size_t)l * N + j) * K + kk] : 0;
+        const uint64_t v = kk < K ? op[((size_t)l * n_op + j) * K + kk] : 0;
         for (uint32_t i = 0; i < r; ++i)
             planes[((size_t)l * r + i) * total + idx] = (int8_t)crt_residue(v, q, k.mod[i], k.wlo[i], k.whi[i], k.inv_m[i]);
     }
@@ -339,7 +339,7 @@ __global__ void __launch_bounds__(256) k_crt_planes_i8(const uint64_t *op, int8_
 // of the last 256-column tile).  One thread per (column, 8 consecutive k): it reads 64 bytes of
 // the operand and writes one 16-byte core-matrix row per modulus; consecutive threads take
 // consecutive columns, so their stores fill contiguous memory.
-__global__ void __launch_bounds__(256) k_crt_planes_f16(const uint64_t *op, __half *planes, uint64_t N, uint64_t K,
+__global__ void __launch_bounds__(256) k_crt_planes_f16(const uint64_t *op, uint64_t n_op, __half *planes, uint64_t N, uint64_t K,
                                                         uint64_t Kp, icm::I8Consts k) {
     const uint32_t l = blockIdx.y;
     const uint32_t r = k.n_mod;
@@ -349,7 +349,7 @@ __global__ void __launch_bounds__(256) k_crt_planes_f16(const uint64_t *op, __ha
         const uint64_t j = idx % Np, k0 = (idx / Np) * 8;
         uint64_t v[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) v[e] = (j < N && k0 + e < K) ? op[((size_t)l * N + j) * K + k0 + e] : 0;
+        for (int e = 0; e < 8; ++e) v[e] = (j < N && k0 + e < K) ? op[((size_t)l * n_op + j) * K + k0 + e] : 0;
         const uint64_t o = icm::crt_f16_off(j, k0, N, Kp);
         for (uint32_t i = 0; i < r; ++i) {
             uint32_t w[4];
@@ -420,14 +420,14 @@ bool make_chunk_tab(const uint64_t *const *A, uint64_t *const *C, const uint64_t
     return true;
 }
 
-cudaError_t launch_crt_planes(bool f16, const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K,
-                              uint64_t Kp, cudaStream_t st) {
+cudaError_t launch_crt_planes(bool f16, const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N,
+                              uint64_t K, uint64_t Kp, cudaStream_t st) {
     if (N == 0 || Kp == 0) return cudaSuccess;
     if (Kp % 16 || (f16 && reinterpret_cast<uintptr_t>(planes) % 16)) return cudaErrorInvalidValue;
     const uint64_t total = f16 ? crt_f16_ncols(N) * (Kp / 8) : N * Kp;
     const unsigned blocks = (unsigned)std::min<uint64_t>((total + 255) / 256, 152u * 32u);
-    if (f16) k_crt_planes_f16<<<dim3(blocks, k.n_limbs), 256, 0, st>>>(op, reinterpret_cast<__half *>(planes), N, K, Kp, k);
-    else k_crt_planes_i8<<<dim3(blocks, k.n_limbs), 256, 0, st>>>(op, reinterpret_cast<int8_t *>(planes), N, K, Kp, k);
+    if (f16) k_crt_planes_f16<<<dim3(blocks, k.n_limbs), 256, 0, st>>>(op, n_op, reinterpret_cast<__half *>(planes), N, K, Kp, k);
+    else k_crt_planes_i8<<<dim3(blocks, k.n_limbs), 256, 0, st>>>(op, n_op, reinterpret_cast<int8_t *>(planes), N, K, Kp, k);
     return cudaGetLastError();
 }
 
@@ -454,7 +454,8 @@ cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const C
     if (Mall == 0 || N == 0) return cudaSuccess;
     // limbs in groups that fit the residue scratch: each group is the same product on a slice of
     // the database words, query planes and outputs
-    const uint32_t G = crt_limb_group(k.n_limbs, k.n_mod, N, Mall);
+    const uint64_t n_out = tab.n_out ? tab.n_out : N;                    // the scratch is sized for these
+    const uint32_t G = crt_limb_group(k.n_limbs, k.n_mod, n_out, Mall);
     if (G < k.n_limbs) {
         const uint64_t plane_limb = crt_plane_bytes(f16, 1, k.n_mod, N, Kp);
         for (uint32_t l0 = 0; l0 < k.n_limbs; l0 += G) {
@@ -462,7 +463,7 @@ cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const C
             ChunkTab t = tab;
             for (uint32_t c = 0; c < tab.n; ++c) {
                 t.A[c] = tab.A[c] + (uint64_t)l0 * tab.M[c] * K;
-                t.C[c] = tab.C[c] + (uint64_t)l0 * N * tab.M[c];
+                t.C[c] = tab.C[c] + (uint64_t)l0 * n_out * tab.M[c];
             }
             const I8Consts s = limb_slice(k, l0, n);
             cudaError_t e = launch_ppmm_crt_grouped(f16, bn, s, t, static_cast<const char *>(Bp) + l0 * plane_limb, N,
@@ -496,7 +497,7 @@ cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const C
 cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const void *scratch, uint64_t N, uint64_t n0,
                                uint64_t nch, cudaStream_t st) {
     const uint64_t Mall = tab.row0[tab.n];
-    P2Args b{tab, reinterpret_cast<const uint8_t *>(scratch), N, n0, nch, k};
+    P2Args b{tab, reinterpret_cast<const uint8_t *>(scratch), tab.n_out ? tab.n_out : N, n0, nch, k};
     if ((Mall & 3) == 0) {
         const uint64_t threads = nch * Mall / 4;
         k_crt_combine<4><<<dim3((unsigned)((threads + 255) / 256), k.n_limbs), 256, 0, st>>>(b);

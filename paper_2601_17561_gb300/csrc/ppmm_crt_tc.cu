@@ -47,8 +47,8 @@
 //    and one commit to both blocks.  The leader's "full" barrier of a stage counts the converter
 //    warps of both blocks and the bytes of both blocks' planes;
 //  * epilogue (8 warps per block, two per TMEM lane quarter): reduces an accumulator in place
-//    (tcgen05.ld / st) at its reduction points or writes the final residues, 16 database rows of
-//    one query column per thread as one 16-byte store.  The accumulators' reduction points are
+//    (tcgen05.ld / st) at its reduction points or writes the final residues, 64 database rows of
+//    one query column per thread.  The accumulators' reduction points are
 //    staggered by a quarter of the interval; the issuer goes on with the others while one is
 //    reduced and catches up when it is back.
 // Option SYNC (cooperative launch): the pairs start fetching the operands of their w-th tile only
@@ -84,7 +84,8 @@ constexpr int FLUSH_K = 1024;                     // columns of K between reduct
 constexpr int NCG = 4, WPG = 2, NCV = NCG * WPG;  // converter groups, warps per group
 constexpr int ROWS_W = ROWS / WPG, ITEMS = ROWS_W / 16;   // rows of a converter warp, in items of 16
 constexpr int NEP = 8;                            // epilogue warps: two per TMEM lane quarter
-constexpr int EP_COLS = BM / 2;                   // accumulator columns of one epilogue warp
+constexpr int EP_COLS = BM / 2;                   // accumulator columns (database rows) of one epilogue warp
+static_assert(EP_COLS == 64, "store_residues");
 constexpr uint64_t LAUNCH_COLS = 1024;            // columns of one launch: the scratch width
 
 // Configuration of a launch: G column groups of 256 x NM moduli per tile, S operand stages of KH slabs,
@@ -374,6 +375,28 @@ __device__ __forceinline__ uint32_t res_pair(uint64_t z0, uint64_t z1, const Res
     return out;
 }
 
+// Writes the first n (0..64) of a thread's 64 bytes to an address of any alignment: whole rows as 4-byte
+// words with bytes at the edges.  (64 single bytes, each a 32-line store of the warp, took the epilogue
+// 16,000 cycles per accumulator: 8 eyes against three chunks of odd sizes 20.8 -> 18.5 ms.)
+__device__ __forceinline__ void store_residues(uint8_t *d, const uint32_t (&w)[16], uint32_t n) {
+    if (n == 64) {
+        const uint32_t head = (4u - (uint32_t)(reinterpret_cast<uintptr_t>(d) & 3)) & 3u;   // bytes before the first whole word
+        uint32_t *q = reinterpret_cast<uint32_t *>(d + head);
+#pragma unroll
+        for (int i = 0; i < 15; ++i) q[i] = __funnelshift_r(w[i], w[i + 1], 8 * head);
+        if (head == 0) {
+            q[15] = w[15];
+        } else {
+            for (uint32_t i = 0; i < head; ++i) d[i] = (uint8_t)(w[0] >> (8 * i));
+            for (uint32_t i = head; i < 4; ++i) d[60 + i] = (uint8_t)(w[15] >> (8 * i));
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 64; ++i)
+            if ((uint32_t)i < n) d[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+    }
+}
+
 template <class C>
 struct __align__(8) Bars {
     // raw slots; operand stages (planes and residues; "full" is used in the leader only); per
@@ -614,13 +637,11 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
                     }
                     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                 } else {
-#pragma unroll 1
-                    for (uint32_t c = 0; c < EP_COLS / 16; ++c) {
+                    // residues in [0, m) of 16 database rows as bytes (the float's low mantissa bits, r + 2^23)
+                    auto chunk = [&](uint32_t c, uint32_t *w) {
                         uint32_t va[16];
                         tmem_ld<16>(tbase + c * 16, va);
                         reduce(va);
-                        // residues in [0, m) as bytes of the float's low mantissa bits (r + 2^23)
-                        uint32_t w[4];
 #pragma unroll
                         for (int i = 0; i < 16; ++i) {
                             const float r = __uint_as_float(va[i]);
@@ -630,15 +651,28 @@ __global__ void __launch_bounds__(C::NTHREADS, 1) k_crt_tc(const __grid_constant
                         for (int i = 0; i < 4; ++i)
                             w[i] = __byte_perm(__byte_perm(va[4 * i], va[4 * i + 1], 0x0040),
                                                __byte_perm(va[4 * i + 2], va[4 * i + 3], 0x0040), 0x5410);
-                        const uint64_t row = row0 + c * 16;
-                        uint8_t *d = dst + c * 16;
-                        if (col_ok && row + 16 <= tc.M && (reinterpret_cast<uintptr_t>(d) & 15) == 0) {
-                            *reinterpret_cast<uint4 *>(d) = make_uint4(w[0], w[1], w[2], w[3]);
-                        } else if (col_ok) {
+                    };
+                    const uint32_t rows = col_ok && row0 < tc.M ? (uint32_t)min((uint64_t)EP_COLS, tc.M - row0) : 0u;
+                    if (((reinterpret_cast<uintptr_t>(p.R) | Mall | p.tab.row0[tc.c]) & 15) == 0) {
+                        // every column's rows start on 16 bytes
+#pragma unroll 1
+                        for (uint32_t c = 0; c < EP_COLS / 16; ++c) {
+                            uint32_t w[4];
+                            chunk(c, w);
+                            if (rows >= (c + 1) * 16) {
+                                *reinterpret_cast<uint4 *>(dst + c * 16) = make_uint4(w[0], w[1], w[2], w[3]);
+                            } else {
 #pragma unroll
-                            for (int i = 0; i < 16; ++i)
-                                if (row + i < tc.M) d[i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+                                for (uint32_t i = 0; i < 16; ++i)
+                                    if (c * 16 + i < rows) dst[c * 16 + i] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
+                            }
+                            __syncwarp();
                         }
+                    } else {
+                        uint32_t w[EP_COLS / 4];
+#pragma unroll
+                        for (uint32_t c = 0; c < EP_COLS / 16; ++c) chunk(c, w + 4 * c);
+                        store_residues(dst, w, rows);
                         __syncwarp();
                     }
                 }
@@ -903,22 +937,24 @@ cudaError_t crt_tc_set_attributes() {
     return e;
 }
 
-// The digit form takes the fp16 form's product where its planes fit the residue planes' place in the
-// operand (so that buffer sizes do not depend on the choice): up to n_mod / 8 groups of 32 columns,
-// 2 for 60-bit primes, and at most 64 columns.  There one pass of a row tile per group costs 2,048
-// cycles per 16 words and 256 rows, the CRT kernel's conversions 5,500 to 7,400 for any width up to
-// 256 columns (measured: 1 eye x 3,000 codes, 8 limbs: 3.8 ms against 13.1; the product of 2 eyes x 8,192 rows 7.2 against 14.7).
-uint32_t dig_groups(uint32_t n_mod, uint64_t N, uint64_t K) {
-    const uint64_t g = (N + 31) / 32;
-    return N > 0 && g <= 2 && g * 8 <= n_mod && crt_tc_supported(K) ? (uint32_t)g : 0;
+// The digit form takes the columns that would leave the last group of 256 nearly empty, where its planes
+// fit the residue planes' place in the operand (so that buffer sizes do not depend on the choice): up to
+// n_mod / 8 groups of 32 columns, 2 for 60-bit primes.  One pass of a row tile per group costs 2,048 cycles
+// per 16 words and 256 rows whatever the rest.  Measured for 8,192 rows and 8 limbs (ms): digits 3.6 per
+// group; residues 13.2, 19.9, 33.4, 40.3 for one to four groups of 256.  So one group of 32 always
+// goes to the digits, two where the last group of 256 would be the first or third of its launch.
+uint32_t dig_cols(uint32_t n_mod, uint64_t N, uint64_t K) {
+    const uint32_t rem = (uint32_t)(N % 256), g = (rem + 31) / 32;
+    const bool pays = g == 1 || (g == 2 && (N / 256) % 2 == 0);
+    return pays && g * 8 <= n_mod && crt_tc_supported(K) ? rem : 0;
 }
 
-cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K, uint64_t Kp,
-                              cudaStream_t st) {
+cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N, uint64_t K,
+                              uint64_t Kp, cudaStream_t st) {
     if (reinterpret_cast<uintptr_t>(planes) % 16) return cudaErrorInvalidValue;
     DigPlanesArgs a{};
     a.op = op; a.planes = reinterpret_cast<unsigned char *>(planes);
-    a.N = N; a.K = K; a.Kp = Kp; a.groups = dig_groups(k.n_mod, N, K);
+    a.n_op = n_op; a.N = N; a.K = K; a.Kp = Kp; a.groups = (uint32_t)((N + 31) / 32);
     for (uint32_t l = 0; l < k.n_limbs; ++l) {
         a.q[l] = k.q[l];
         for (int t = 0; t < 8; ++t) { a.w[l][t] = k.pw8[l][t]; a.ws[l][t] = k.pw8s[l][t]; }
@@ -928,8 +964,8 @@ cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, void *plane
     return cudaGetLastError();
 }
 
-cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
-                            cudaStream_t st) {
+cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t col0, uint64_t N, uint64_t K,
+                            uint64_t Kp, cudaStream_t st) {
     if (tab.row0[tab.n] == 0 || N == 0) return cudaSuccess;
     if (!crt_tc_aligned(tab) || reinterpret_cast<uintptr_t>(Bp) % 16) return cudaErrorInvalidValue;
     EncodeTiled enc = encode_fn();
@@ -950,7 +986,7 @@ cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *
             return cudaErrorInvalidValue;
         a.t0[c + 1] = a.t0[c] + (uint32_t)((tab.M[c] + DG_TILE - 1) / DG_TILE);
     }
-    a.groups = dig_groups(k.n_mod, N, K);
+    a.groups = (uint32_t)((N + 31) / 32);
     const cuuint64_t dims[2] = {256, (cuuint64_t)k.n_limbs * a.groups * 2 * Kp}, strides[1] = {2048};
     const cuuint32_t box[2] = {256, DG_WORDS};
     if (enc(&a.tmB, CU_TENSOR_MAP_DATA_TYPE_UINT64, 2, const_cast<void *>(Bp), dims, strides, box, estr,
@@ -958,7 +994,7 @@ cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
         return cudaErrorInvalidValue;
     a.tab = tab;
-    a.N = N; a.K = K; a.Kp = Kp; a.n_limbs = k.n_limbs;
+    a.N = N; a.K = K; a.Kp = Kp; a.n_limbs = k.n_limbs; a.col0 = col0; a.n_out = tab.n_out ? tab.n_out : N;
     a.n_tiles = (uint64_t)k.n_limbs * a.t0[tab.n] * a.groups;
     a.wait_ns = k.tc_wait_ns ? k.tc_wait_ns : 2000000000ull;
     a.inject_stall = k.tc_inject_stall;

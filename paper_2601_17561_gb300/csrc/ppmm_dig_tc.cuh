@@ -40,7 +40,8 @@ struct DigArgs {
     CUtensorMap tmB;                  // digit planes as rows of 2 KB: [L][groups][2][Kp]
     icm::ChunkTab tab;
     uint32_t t0[ICM_MAX_CHUNKS + 1];  // prefix sums of 256-row tiles
-    uint64_t N, K, Kp;
+    uint64_t N, K, Kp;                // query columns of this product
+    uint64_t col0, n_out;             // their first column in the outputs, columns of the outputs
     uint32_t n_limbs, groups;         // column groups of 32
     uint64_t n_tiles;                 // L x row tiles x groups
     uint64_t wait_ns;
@@ -249,7 +250,7 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dig_tc(const __grid_constant_
                             }
                             const uint64_t col = (uint64_t)tc.g * 32 + half * 16 + 4 * x + n;
                             if (row < tc.M && col < p.N)
-                                p.tab.C[tc.c][((size_t)tc.l * p.N + col) * tc.M + row] =
+                                p.tab.C[tc.c][((size_t)tc.l * p.n_out + p.col0 + col) * tc.M + row] =
                                     add_mod(reduce_s64(lo, q, r64), mulmod_shoup(reduce_s64(hi, q, r64), p.p32[tc.l], p.p32s[tc.l], q), q);
                         }
                         __syncwarp();
@@ -371,9 +372,9 @@ __global__ void __launch_bounds__(DG_THREADS, 1) k_dig_tc(const __grid_constant_
 // warp's stores fill 512 contiguous bytes.  Bound by those stores (128 bytes per operand word): 1 eye, 8
 // limbs, 805 MB in 162 us (494 us with a word per lane, whose stores were 128 bytes apart).
 struct DigPlanesArgs {
-    const uint64_t *op;               // [L][N][K] canonical
+    const uint64_t *op;               // first column of [L][n_op][K] canonical residues
     unsigned char *planes;
-    uint64_t N, K, Kp;
+    uint64_t n_op, N, K, Kp;
     uint32_t groups;
     uint64_t q[ICM_MAX_LIMBS], w[ICM_MAX_LIMBS][8], ws[ICM_MAX_LIMBS][8];    // 256^t mod q, Shoup companions
 };
@@ -386,7 +387,7 @@ __global__ void __launch_bounds__(256) k_dig_planes(const __grid_constant__ DigP
         const uint64_t y = x >> 3, k0 = (y % n_oct) * 8;
         const uint32_t g = (uint32_t)(y / n_oct), nl = (uint32_t)(x & 7) * 4 + sub;   // column of the group
         const uint64_t n = (uint64_t)g * 32 + nl;
-        const uint64_t *src = a.op + ((size_t)l * a.N + n) * a.K;
+        const uint64_t *src = a.op + ((size_t)l * a.n_op + n) * a.K;
         unsigned char *dst = a.planes + ((((size_t)l * a.groups + g) * 2 + (nl >> 4)) * a.Kp + k0) * DG_BLK + (nl & 15) * 128 + t * 16;
         for (uint32_t i = 0; i < 8; ++i) {
             const uint64_t v = (n < a.N && k0 + i < a.K) ? __ldg(src + k0 + i) : 0;

@@ -46,11 +46,12 @@ cudaError_t launch_planes(int form, const I8Consts &k, const uint64_t *op, int8_
 struct ChunkTab {
     uint32_t n;
     const uint64_t *A[ICM_MAX_CHUNKS];     // [L][M_c][K]
-    uint64_t *C[ICM_MAX_CHUNKS];           // [L][N][M_c]
+    uint64_t *C[ICM_MAX_CHUNKS];           // [L][n_out][M_c]
     uint64_t M[ICM_MAX_CHUNKS];
     uint64_t row0[ICM_MAX_CHUNKS + 1];     // prefix sums of M_c
     uint32_t mt0[ICM_MAX_CHUNKS + 1];      // prefix sums of 128-row tiles
     int a_digits;                          // A in the balanced-digit storage form (else canonical)
+    uint64_t n_out;                        // columns of the outputs C (0: those of the product)
 };
 bool make_chunk_tab(const uint64_t *const *A, uint64_t *const *C, const uint64_t *M, uint32_t n, ChunkTab &t);
 cudaError_t launch_ppmm_crt_grouped(bool f16, int bn, const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N,
@@ -68,13 +69,14 @@ cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const voi
 cudaError_t crt_tc_set_attributes();
 bool crt_tc_supported(uint64_t K);
 bool crt_tc_aligned(const ChunkTab &tab);
-// Digit form of the fp16 product for few columns (ppmm_dig_tc.cuh): column groups of 32, or 0 where the
-// CRT form is taken; its planes lie where the residue planes would.
-uint32_t dig_groups(uint32_t n_mod, uint64_t N, uint64_t K);
-cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K, uint64_t Kp,
-                              cudaStream_t st);
-cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
-                            cudaStream_t st);
+// Digit form of the fp16 product (ppmm_dig_tc.cuh): how many of the last columns of N it takes (0: none);
+// its planes follow the residue planes of the others, within their place for N columns.  The planes are
+// made from n columns at `op` of an operand of n_op columns; the product writes columns col0 ...
+uint32_t dig_cols(uint32_t n_mod, uint64_t N, uint64_t K);
+cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N, uint64_t K,
+                              uint64_t Kp, cudaStream_t st);
+cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t col0, uint64_t N, uint64_t K,
+                            uint64_t Kp, cudaStream_t st);
 cudaError_t launch_ppmm_crt_tc(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t N, uint64_t K, uint64_t Kp,
                                void *scratch, int variant, cudaStream_t st);
 uint32_t device_status(bool clear);
@@ -119,8 +121,8 @@ inline uint64_t crt_scratch_main_bytes(uint32_t n_limbs, uint32_t n_mod, uint64_
     return (crt_limb_group(n_limbs, n_mod, N, M) * per + 255) / 256 * 256;
 }
 uint64_t crt_scratch_bytes(uint32_t n_limbs, uint32_t n_mod, uint64_t N, uint64_t M);
-cudaError_t launch_crt_planes(bool f16, const I8Consts &k, const uint64_t *op, void *planes, uint64_t N, uint64_t K,
-                              uint64_t Kp, cudaStream_t st);
+cudaError_t launch_crt_planes(bool f16, const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N,
+                              uint64_t K, uint64_t Kp, cudaStream_t st);
 cudaError_t launch_ppmm_crt(bool f16, int bn, const I8Consts &k, const uint64_t *A, bool a_digits, const void *Bp,
                             uint64_t *C, uint64_t M, uint64_t N, uint64_t K, uint64_t Kp, void *scratch, cudaStream_t st);
 cudaError_t launch_ppmm_i8(int form, const I8Consts &k, const uint64_t *A, bool a_digits, const int8_t *Bp, uint64_t *C,

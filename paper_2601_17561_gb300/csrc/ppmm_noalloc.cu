@@ -112,7 +112,7 @@ extern "C" icm_status icm_ppmm_noalloc(icm_form form, const uint64_t *q, uint32_
         }
     }
     cudaStream_t st = (cudaStream_t)stream;
-    e = launch_crt_planes(f16, k, dev_B, ws, N, K, Kp, st);
+    e = launch_crt_planes(f16, k, dev_B, N, ws, N, K, Kp, st);
     if (e == cudaSuccess)
         e = launch_ppmm_crt(f16, 256, k, dev_A, false, ws, dev_C, M, N, K, Kp, (char *)ws + a256(planes), st);
     if (e != cudaSuccess) return api_fail(ICM_ECUDA, cudaGetErrorString(e));

@@ -19,22 +19,22 @@ def setup():
     # 56-bit primes: 17 CRT moduli
     eng = E.Engine(**{**E.TINY, "log_n_db": 7, "prime_bits": 56, "seed": 6}, hamming_weight=64).keygen()
     assert len(C.icm_ctx_crt_moduli(eng.ctx)) == 17
-    W = synth.make_workload(n_eyes=26, n_db=231, seed=31)
+    W = synth.make_workload(n_eyes=34, n_db=231, seed=31)
     cuts = [0, 1, 150, 231]
     dbs = [eng.encrypt_db(W.db_codes[a:b], W.db_masks[a:b], chunk_id=i) for i, (a, b) in enumerate(zip(cuts, cuts[1:]))]
     return eng, W, dbs
 
 
-@pytest.mark.parametrize("n_eyes", [1, 8, 9, 16, 17, 24, 25])
+@pytest.mark.parametrize("n_eyes", [1, 8, 9, 16, 17, 18, 24, 25, 34])
 def test_column_groups(setup, n_eyes):
     eng, W, dbs = setup
     ct = eng.encrypt_query(W.q_codes[:n_eyes], W.q_masks[:n_eyes], W.eye_ids[:n_eyes])
-    q = eng.prepare(ct, n_eyes, "f16_crt")
     res = {}
     try:
         for v in (256, 1, 2, 3):
             C.icm_ctx_set_variant(eng.ctx, v)
-            outs = eng.match_batch(dbs, q)
+            # columns just past a multiple of 256 (9, 17, 18, 25, 34 eyes) go to the digit planes on tcgen05
+            outs = eng.match_batch(dbs, eng.prepare(ct, n_eyes, "f16_crt"))
             torch.cuda.synchronize()
             res[v] = [s.residues() for s in outs]
     finally:
