@@ -204,7 +204,9 @@ icm_status icm_ctx_create(const icm_params *p, icm_ctx **out) {
     c->crt_q = c->crt;
     c->rs = icm::RescaleConsts{};
     c->rs.L = P.n_limbs; c->rs.Lq = P.n_limbs_q;
-    for (uint32_t l = 0; l < P.n_limbs; ++l) c->rs.q[l] = q[l];
+    for (uint32_t l = 0; l < P.n_limbs; ++l) {
+        c->rs.q[l] = q[l]; c->rs.rhi[l] = c->crt.rhi[l]; c->rs.rlo[l] = c->crt.rlo[l];
+    }
     for (uint32_t l = 0; l < P.n_limbs_q; ++l) {
         uint64_t hat = 1 % q[l];
         for (uint32_t j = 0; j < P.n_limbs_q; ++j) if (j != l) hat = mulmod(hat, q[j] % q[l], q[l]);
@@ -216,19 +218,17 @@ icm_status icm_ctx_create(const icm_params *p, icm_ctx **out) {
         for (uint32_t k = P.n_limbs_q; k < P.n_limbs; ++k) if (k != i) hat = mulmod(hat, q[k] % q[i], q[i]);
         c->rs.yinv[i] = powmod(hat, q[i] - 2, q[i]);
         c->rs.yinvs[i] = shoup_of(c->rs.yinv[i], q[i]);
-        c->rs.rhi[i] = c->crt.rhi[i]; c->rs.rlo[i] = c->crt.rlo[i];
     }
     for (uint32_t j = 0; j < P.n_limbs_q; ++j) {
         uint64_t qp = 1 % q[j];
+        for (uint32_t i = P.n_limbs_q; i < P.n_limbs; ++i) qp = mulmod(qp, q[i] % q[j], q[j]);
+        c->rs.qpinv[j] = powmod(qp, q[j] - 2, q[j]);
         for (uint32_t i = P.n_limbs_q; i < P.n_limbs; ++i) {
             uint64_t hat = 1 % q[j];
             for (uint32_t k = P.n_limbs_q; k < P.n_limbs; ++k) if (k != i) hat = mulmod(hat, q[k] % q[j], q[j]);
-            c->rs.w[j][i] = hat;
-            c->rs.ws[j][i] = shoup_of(hat, q[j]);
-            qp = mulmod(qp, q[i] % q[j], q[j]);
+            const uint64_t w = mulmod(hat, c->rs.qpinv[j], q[j]);
+            c->rs.w[j][i] = w ? q[j] - w : 0;
         }
-        c->rs.qp[j] = qp; c->rs.qps[j] = shoup_of(qp, q[j]);
-        c->rs.qpinv[j] = powmod(qp, q[j] - 2, q[j]); c->rs.qpinvs[j] = shoup_of(c->rs.qpinv[j], q[j]);
     }
     *out = c;
     return ICM_OK;

@@ -206,15 +206,27 @@ __device__ __forceinline__ void rescale_one(const icm::RescaleConsts &k, const u
         shi += slo < f ? 1 : 0;
     }
     const uint64_t v = shi + ((slo >> 63) & 1);                    // floor((S + 2^63) / 2^64)
+    // x'_j = (x_j - y) Q'^-1 = x_j Q'^-1 + sum_i yh_i w_ji + v mod q_j: one 128-bit sum of products below
+    // 2^123 and one reduction (a Shoup product with its reduction for each term took three 64-bit
+    // products where the sum takes one)
     for (uint32_t j = 0; j < Lq; ++j) {
-        const uint64_t q = k.q[j];
-        uint64_t y = 0;
+        const uint64_t q = k.q[j], x = in[(size_t)j * n + c];
+        uint64_t lo = x * k.qpinv[j], hi = __umul64hi(x, k.qpinv[j]);
+        lo += v;
+        hi += lo < v ? 1 : 0;
 #pragma unroll
         for (uint32_t i = 0; i < ICM_MAX_LIMBS; ++i)
-            if (i >= Lq && i < L) y = add_mod(y, mulmod_shoup(yh[i], k.w[j][i], k.ws[j][i], q), q);
-        y = sub_mod(y, mulmod_shoup(v, k.qp[j], k.qps[j], q), q);
-        const uint64_t d = sub_mod(in[(size_t)j * n + c], y, q);
-        out[(size_t)j * n + c] = mulmod_shoup(d, k.qpinv[j], k.qpinvs[j], q);
+            if (i >= Lq && i < L) {
+                const uint64_t p = yh[i] * k.w[j][i];
+                lo += p;
+                hi += __umul64hi(yh[i], k.w[j][i]) + (lo < p ? 1 : 0);
+            }
+        // the quotient estimate is short by at most 4, so the remainder is below 5 q < 2^63
+        const uint64_t qe = hi * k.rhi[j] + __umul64hi(hi, k.rlo[j]) + __umul64hi(lo, k.rhi[j]);
+        uint64_t r = lo - qe * q;
+        r = r >= 2 * q ? r - 2 * q : r;
+        r = r >= 2 * q ? r - 2 * q : r;
+        out[(size_t)j * n + c] = r >= q ? r - q : r;
     }
 }
 

@@ -30,15 +30,14 @@ struct CrtDecode {               // constants of the fixed-point CRT decoding (d
 };
 
 // Rescaling by Q' (x' = round(x / Q') mod Q, base conversion from the limbs of Q' to those of Q):
-// for the limbs i of Q' (i >= Lq) yinv_i = (Q'/q_i)^-1 mod q_i; for the limbs j of Q (j < Lq)
-// w[j][i] = (Q'/q_i) mod q_j, qp_j = Q' mod q_j and qpinv_j = Q'^-1 mod q_j; Shoup companions.
+// for the limbs i of Q' (i >= Lq) yinv_i = (Q'/q_i)^-1 mod q_i (Shoup companion yinvs); for the limbs j of
+// Q (j < Lq) qpinv_j = Q'^-1 mod q_j and w[j][i] = -(Q'/q_i) Q'^-1 mod q_j.
 struct RescaleConsts {
     uint32_t L, Lq;
     uint64_t q[ICM_MAX_LIMBS];
     uint64_t yinv[ICM_MAX_LIMBS], yinvs[ICM_MAX_LIMBS];
     uint64_t rhi[ICM_MAX_LIMBS], rlo[ICM_MAX_LIMBS];       // floor(2^128 / q_i), high and low words
-    uint64_t w[ICM_MAX_LIMBS][ICM_MAX_LIMBS], ws[ICM_MAX_LIMBS][ICM_MAX_LIMBS];
-    uint64_t qp[ICM_MAX_LIMBS], qps[ICM_MAX_LIMBS], qpinv[ICM_MAX_LIMBS], qpinvs[ICM_MAX_LIMBS];
+    uint64_t w[2][ICM_MAX_LIMBS], qpinv[2];
 };
 
 // Transforms of the rings up to 2^14 (ntt.cuh), on the context's device: tables per limb, and the
