@@ -183,7 +183,10 @@ constexpr int NT_MUL = 512;
 // but a transform costs about 7 Shoup products per coefficient.  Columns are taken four at a time
 // where 2^14 words hold them, so that a row's words fill a 32-byte sector and the columns share
 // their twiddles.  1,000 templates at N_db = 2^12, four primes (4.0 GB): 69.5 ms with the
-// additions, 12.1 ms now (11.4 of them here).
+// additions, 11.6 ms now (11 of them here: 6.6 the transforms, 2.3 the pointwise products, 1 the noise
+// and the rows' update, 0.8 drawing and storing the a-part).  Twice the threads (64 registers, the
+// polynomial kept in shared memory or not at all) or two blocks of half the columns give the same
+// time, one column per block 13.2 ms: multiplications bound it, not latency.
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant__ DbEncArgs a) {
     extern __shared__ uint64_t su[];                                     // [2^logc][stride]
@@ -230,8 +233,8 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant_
             if (k >= a.K || (part && i >= a.lay.rem && i < a.lay.tail_lo)) continue;
             const uint64_t row = (uint64_t)N + (uint64_t)t * N + (part && i >= a.lay.rem ? a.lay.rem + (i - a.lay.tail_lo) : i);
             const uint64_t r = (uint64_t)t * N + i;
-            uint64_t sa = su[c * stride + icm::ntt_pad(i)];              // (s_{db,t} * a)[i], below 2q
-            sa = sa >= q ? sa - q : sa;
+            // (s_{db,t} * a)[i], below 4q
+            const uint64_t sa = icm::sub_if(icm::sub_if(su[c * stride + icm::ntt_pad(i)], 2 * q), q);
             uint64_t *dst = dbl + (size_t)row * a.K + k;
             const int e = cbd_sample(sm64(ke, r * a.K + k), a.eta);
             // messages are multiples of Q', zero modulo the limbs of Q'
@@ -255,33 +258,35 @@ struct QEncArgs {
 };
 
 // One block per (2^logc query columns, limb l < Lq): the same transforms as k_db_apart_b.  32 eyes
-// (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient,
-// 1.26 ms now.
+// (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient, 1.24 ms
+// with the column and eye of each word divided out, 1.01 ms now.
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_constant__ QEncArgs a) {
     extern __shared__ uint64_t su[];                               // [2^logc][stride]
     const uint32_t C = 1u << a.logc, l = blockIdx.y, N = a.Nq, j0 = blockIdx.x << a.logc;
-    const uint32_t stride = icm::ntt_words(N) + 4, CN = N << a.logc;
+    const uint32_t stride = icm::ntt_words(N) + 4, CN = N << a.logc, lgN = 31 - __clz(N);
     const uint64_t q = a.q[l];
     const icm::NttMod &T = a.nt[l];
-    // word x: coefficient x mod N of column x / N
-    for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
-        const uint32_t c = x / N, i = x % N, j = j0 + c;
-        uint64_t v = 0;
-        if (j < a.n_cols) {
-            const uint64_t ka = stream_key(a.seed, ICM_KIND_A_Q, a.eye_ids[j / a.rho], l);
-            v = uniform_mod(sm64(ka, (uint64_t)(j % a.rho) * N + i), q);
-            a.ct[((size_t)l * a.n_cols + j) * a.K + a.d2 + i] = v;
+    for (uint32_t c = 0; c < C; ++c) {
+        const uint32_t j = j0 + c, r = j % a.rho;
+        const uint64_t ka = j < a.n_cols ? stream_key(a.seed, ICM_KIND_A_Q, a.eye_ids[j / a.rho], l) : 0;
+        for (uint32_t i = threadIdx.x; i < N; i += NT_MUL) {
+            uint64_t v = 0;
+            if (j < a.n_cols) {
+                v = uniform_mod(sm64(ka, (uint64_t)r * N + i), q);
+                a.ct[((size_t)l * a.n_cols + j) * a.K + a.d2 + i] = v;
+            }
+            su[c * stride + icm::ntt_pad(i)] = v;
         }
-        su[c * stride + icm::ntt_pad(i)] = v;
     }
     __syncthreads();
     icm::ntt_forward(su, C, stride, N, T);
+    // word x: coefficient x mod N of column x / N
     uint64_t ah[WPT];
 #pragma unroll
     for (int w = 0; w < WPT; ++w) {
         const uint32_t x = threadIdx.x + w * NT_MUL;
-        if (x < CN) ah[w] = su[(x / N) * stride + icm::ntt_pad(x % N)];
+        if (x < CN) ah[w] = su[(x >> lgN) * stride + icm::ntt_pad(x & (N - 1))];
     }
     const uint32_t tb = a.code_bits / 8;
     for (uint32_t t = 0; t < a.nqblk; ++t) {
@@ -290,32 +295,35 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_consta
         for (int w = 0; w < WPT; ++w) {
             const uint32_t x = threadIdx.x + w * NT_MUL;
             if (x < CN)
-                su[(x / N) * stride + icm::ntt_pad(x % N)] = icm::mul_r128_lazy(ah[w], __ldg(sh + x % N), T);
+                su[(x >> lgN) * stride + icm::ntt_pad(x & (N - 1))] = icm::mul_r128_lazy(ah[w], __ldg(sh + (x & (N - 1))), T);
         }
         __syncthreads();
         icm::ntt_inverse(su, C, stride, N, T);
-        for (uint32_t x = threadIdx.x; x < CN; x += NT_MUL) {
-            const uint32_t c = x / N, i = x % N, j = j0 + c, k = t * N + i;
-            if (j >= a.n_cols) continue;
-            const uint32_t e = j / a.rho, r = j % a.rho;
-            uint64_t sa = su[c * stride + icm::ntt_pad(i)];
-            sa = sa >= q ? sa - q : sa;
-            uint64_t v = sa ? q - sa : 0;                          // -(s * a)
-            // rotated masked bit-vector: x_s[row, col, b] = x[row, (col + s) mod 200, b] on 16 x 200 x 4
-            int m = 0;
-            if (k < a.code_bits) {
-                const int shift = (int)r - (int)(a.rho - 1) / 2;
-                const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
-                const uint32_t src = (row * 200 + (uint32_t)(((int)cc + shift + 200) % 200)) * 4 + b;
-                const int cb = template_bit(a.codes + (size_t)e * tb, src), mb = template_bit(a.masks + (size_t)e * tb, src);
-                m = mb - 2 * (cb & mb);
-            }
-            if (m > 0) v = add_mod(v, a.dl[l], q);
-            else if (m < 0) v = sub_mod(v, a.dl[l], q);
+        for (uint32_t c = 0; c < C; ++c) {
+            const uint32_t j = j0 + c, e = j / a.rho, r = j % a.rho;
+            if (j >= a.n_cols) break;
+            const int shift = (int)r - (int)(a.rho - 1) / 2;
+            const uint8_t *code = a.codes + (size_t)e * tb, *mask = a.masks + (size_t)e * tb;
             const uint64_t ke = stream_key(a.seed, ICM_KIND_E_Q, a.eye_ids[e], 0);
-            const int err = cbd_sample(sm64(ke, (uint64_t)r * a.d2 + k), a.eta);
-            v = err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
-            a.ct[((size_t)l * a.n_cols + j) * a.K + k] = v;
+            uint64_t *ct = a.ct + ((size_t)l * a.n_cols + j) * a.K + (size_t)t * N;
+            for (uint32_t i = threadIdx.x; i < N; i += NT_MUL) {
+                const uint32_t k = t * N + i;
+                const uint64_t sa = icm::sub_if(icm::sub_if(su[c * stride + icm::ntt_pad(i)], 2 * q), q);
+                uint64_t v = sa ? q - sa : 0;                      // -(s * a)
+                // rotated masked bit-vector: x_s[row, col, b] = x[row, (col + s) mod 200, b] on 16 x 200 x 4
+                int m = 0;
+                if (k < a.code_bits) {
+                    const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
+                    const uint32_t src = (row * 200 + (uint32_t)(((int)cc + shift + 200) % 200)) * 4 + b;
+                    const int cb = template_bit(code, src), mb = template_bit(mask, src);
+                    m = mb - 2 * (cb & mb);
+                }
+                if (m > 0) v = add_mod(v, a.dl[l], q);
+                else if (m < 0) v = sub_mod(v, a.dl[l], q);
+                const int err = cbd_sample(sm64(ke, (uint64_t)r * a.d2 + k), a.eta);
+                v = err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
+                ct[i] = v;
+            }
         }
     }
 }

@@ -288,7 +288,7 @@ struct FwdArgs {
     const uint64_t *src; uint64_t src_ls, src_ps;
     uint64_t *dst; uint64_t dst_ls, dst_ps;
 };
-__global__ void __launch_bounds__(512) k_ntt_fwd(const __grid_constant__ FwdArgs a) {
+__global__ void __launch_bounds__(512, 2) k_ntt_fwd(const __grid_constant__ FwdArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t total = (uint64_t)a.Lq * a.per_limb;
     for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
@@ -301,19 +301,16 @@ __global__ void __launch_bounds__(512) k_ntt_fwd(const __grid_constant__ FwdArgs
         __syncthreads();
         icm::ntt_forward(su, 1, 0, a.N, T);
         uint64_t *dd = a.dst + l * a.dst_ls + p * a.dst_ps;
-        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) {
-            uint64_t v = su[icm::ntt_pad(i)];                            // below 4q
-            v = v >= 2 * q ? v - 2 * q : v;
-            dd[i] = v >= q ? v - q : v;
-        }
+        for (uint32_t i = threadIdx.x; i < a.N; i += blockDim.x) dd[i] = icm::ntt_canon(su[icm::ntt_pad(i)], q);
         __syncthreads();
     }
 }
 
 // Output (limb l, column j, block t, part h): part 0 = a_j mu_{j,t}, part 1 = b_{j,t} mu_{j,t};
 // a_ntt holds NTT(a_j), mu_ntt NTT(mu_{j,t}); b rows are read from the rescaled scores.  The
-// transforms' integer products bound it; with three levels per pass over shared memory (ntt.cuh) the
-// normalisation of 8 eyes x 4,096 templates (N_db = 2^13) takes 717 us, 820 us with one level per pass.
+// transforms' integer products bound it; with three levels per pass over shared memory (ntt.cuh) and two
+// blocks per SM (64 registers) the normalisation of 8 eyes x 4,096 templates (N_db = 2^13) takes 652 us,
+// 738 us with one block, 820 us with one level per pass.
 struct MulArgs {
     icm::NttMod nt[2];
     uint32_t N, Lq, n_cols, n_blocks;
@@ -323,7 +320,7 @@ struct MulArgs {
     const uint64_t *mu_ntt;         // [Lq][n_cols][n_blocks][N]
     uint64_t *out;                  // [Lq][n_cols][n_blocks][2][N]
 };
-__global__ void __launch_bounds__(512) k_ntt_mul_inv(const __grid_constant__ MulArgs a) {
+__global__ void __launch_bounds__(512, 2) k_ntt_mul_inv(const __grid_constant__ MulArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t per_limb = (uint64_t)a.n_cols * a.n_blocks * 2;
     const uint64_t total = (uint64_t)a.Lq * per_limb;
