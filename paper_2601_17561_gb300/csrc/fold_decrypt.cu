@@ -96,7 +96,6 @@ struct DecArgs {
     int64_t *num;          // [n_cols][n_real]
     uint32_t *err_bits;    // optional: max |x - round(x)| over all outputs, as fp32 bits
 };
-constexpr int NT_DEC = 512;
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -110,42 +109,48 @@ __device__ __forceinline__ uint64_t ld_cluster(uint32_t addr, uint32_t rank) {
 }
 
 // One cluster of L blocks per column, one block per limb: the transform of the column's a-part stays
-// in registers, and per b-block t a pointwise product and one inverse transform give s_{db,t} * C_a
-// (ntt.cuh); every block then holds its limb's y in shared memory, and the cluster combines the limbs
-// of each coefficient through distributed shared memory, so no limb goes through global memory.
-// Integer products bound it (about 8 per coefficient and limb; the direct form added h = 512 terms
-// per coefficient, from L2).  8 eyes x 3,000 codes, 8 limbs, N_db = 2^12: 4.30 ms with the direct
-// form, 0.40 ms now.
-template <int WPT>
-__global__ void __launch_bounds__(NT_DEC, 1) k_decrypt(const __grid_constant__ DecArgs a) {
+// in registers (WPT words per thread, WPT NT >= N; WPT = 0 where one b-block follows, which takes the
+// transform where it lies), and per b-block t a pointwise product and one inverse transform give
+// s_{db,t} * C_a (ntt.cuh); every block then holds its limb's y in shared memory, and the cluster
+// combines the limbs of each coefficient through distributed shared memory, so no limb goes through
+// global memory.  Integer products bound it (about 8 per coefficient and limb; the direct form added
+// h = 512 terms per coefficient, from L2).  8 eyes x 3,000 codes, 8 limbs, N_db = 2^12: 4.30 ms with
+// the direct form, 0.40 ms with one block of 512 threads per SM, 0.21 ms now.
+template <int WPT, int NT, int MB>
+__global__ void __launch_bounds__(NT, MB) k_decrypt(const __grid_constant__ DecArgs a) {
     extern __shared__ uint64_t su[];
     const uint32_t l = blockIdx.x, j = blockIdx.y, N = a.lay.N;        // block rank in the cluster = limb
     const icm::NttMod &T = a.nt[l];
     const uint64_t q = T.q;
     const uint64_t *col = a.sc + ((size_t)l * a.n_cols + j) * a.lay.M;
     const uint32_t su_addr = (uint32_t)__cvta_generic_to_shared(su);
-    for (uint32_t i = threadIdx.x; i < N; i += NT_DEC) su[icm::ntt_pad(i)] = col[i];
+    for (uint32_t i = threadIdx.x; i < N; i += NT) su[icm::ntt_pad(i)] = col[i];
     __syncthreads();
     icm::ntt_forward(su, 1, 0, N, T);
-    uint64_t ah[WPT];
+    uint64_t ah[WPT ? WPT : 1];
 #pragma unroll
     for (int w = 0; w < WPT; ++w) {
-        const uint32_t i = threadIdx.x + w * NT_DEC;
+        const uint32_t i = threadIdx.x + w * NT;
         if (i < N) ah[w] = su[icm::ntt_pad(i)];
     }
     const uint32_t blocks = (uint32_t)((a.lay.n_real + N - 1) / N);
     for (uint32_t t = 0; t < blocks; ++t) {
         const uint64_t *sh = a.shat + ((size_t)t * a.shat_L + l) * N;
+        if (WPT == 0)
+            for (uint32_t i = threadIdx.x; i < N; i += NT) {
+                uint64_t *w = su + icm::ntt_pad(i);
+                *w = icm::mul_r128_lazy(*w, __ldg(sh + i), T);
+            }
 #pragma unroll
         for (int w = 0; w < WPT; ++w) {
-            const uint32_t i = threadIdx.x + w * NT_DEC;
+            const uint32_t i = threadIdx.x + w * NT;
             if (i < N) su[icm::ntt_pad(i)] = icm::mul_r128_lazy(ah[w], __ldg(sh + i), T);
         }
         __syncthreads();
         icm::ntt_inverse(su, 1, 0, N, T);
         const uint64_t r0 = (uint64_t)t * N;
         const uint32_t rows = (uint32_t)min((uint64_t)N, a.lay.n_real - r0);
-        for (uint32_t i = threadIdx.x; i < rows; i += NT_DEC) {
+        for (uint32_t i = threadIdx.x; i < rows; i += NT) {
             // (s_{db,t} * C_a)[i], below 4q
             const uint64_t sa = icm::sub_if(icm::sub_if(su[icm::ntt_pad(i)], 2 * q), q);
             const uint64_t d = add_mod(col[pos_of(a.lay, (int)t, i)], sa, q);
@@ -153,7 +158,7 @@ __global__ void __launch_bounds__(NT_DEC, 1) k_decrypt(const __grid_constant__ D
         }
         __syncwarp();
         cluster_barrier();
-        for (uint32_t i = l * NT_DEC + threadIdx.x; i < rows; i += a.L * NT_DEC) {
+        for (uint32_t i = l * NT + threadIdx.x; i < rows; i += a.L * NT) {
             uint64_t fhi = 0, flo = 0;                  // sum_l y_l floor(2^128 / q_l) mod 2^128
             for (uint32_t k = 0; k < a.L; ++k) {
                 const uint64_t y = ld_cluster(su_addr + icm::ntt_pad(i) * 8, k);
@@ -279,20 +284,29 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
     if (n_cols == 0 || lay.n_real == 0) return cudaSuccess;
     if (!a.shat) return cudaErrorInvalidValue;                           // rings above 2^14
     const size_t smem = (size_t)ntt_words(lay.N) * 8;
-    auto run = [&](auto kern) {
+    auto run = [&](auto kern, int nt) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
-        cfg.gridDim = dim3(a.L, n_cols); cfg.blockDim = dim3(NT_DEC);
+        cfg.gridDim = dim3(a.L, n_cols); cfg.blockDim = dim3(nt);
         cfg.dynamicSmemBytes = smem; cfg.stream = st;
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = a.L; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         return cudaLaunchKernelEx(&cfg, kern, a);
     };
-    const uint32_t wpt = (lay.N + NT_DEC - 1) / NT_DEC;
-    return wpt > 16 ? run(k_decrypt<32>) : wpt > 8 ? run(k_decrypt<16>) : run(k_decrypt<8>);
+    // Blocks per SM hide the waits at the cluster's barriers.  One b-block: nothing is kept in registers,
+    // and 64 registers a thread allow 1,024 threads per SM, in blocks as small as shared memory lets that
+    // many be resident (248 columns, four limbs: N = 2^12 131 / 143 / 168 us with blocks of 256 / 512 /
+    // 1,024, 2^13 282 / 268 / 317, 2^14 869 / 642 / 573).  Several b-blocks: the transformed a-part takes
+    // N / NT words of registers (2^12 236 us with 256 threads, 311 with 512; 2^13 523 and 594; 2^14 857
+    // with 1,024 threads, 955 with 512).
+    if (lay.n_real <= lay.N)
+        return lay.N <= 4096 ? run(k_decrypt<0, 256, 4>, 256)
+                             : lay.N <= 8192 ? run(k_decrypt<0, 512, 2>, 512) : run(k_decrypt<0, 1024, 1>, 1024);
+    return lay.N <= 4096 ? run(k_decrypt<16, 256, 3>, 256)
+                         : lay.N <= 8192 ? run(k_decrypt<32, 256, 2>, 256) : run(k_decrypt<16, 1024, 1>, 1024);
 }
 
 }  // namespace icm

@@ -58,3 +58,22 @@ def test_decryption_ring_edges(log_n_db, log_n_q, L, Lq, n_db, n_eyes):
     want = O.inner_from_counts(*O.hd_counts(rc, rm, O.unpack(W.db_codes), O.unpack(W.db_masks)))
     assert np.array_equal(eng.decrypt(s).cpu().numpy(), want)
     assert np.array_equal(eng.decrypt(eng.rescale(s)).cpu().numpy(), want)
+
+
+@pytest.mark.parametrize("log_n_db,n_db", [(13, 50), (13, 8250), (14, 50), (14, 16440)])
+def test_decryption_large_rings(log_n_db, n_db):
+    """The block shapes of the larger rings, with one b-block and with a second, partial one."""
+    B.build()
+    prm = dict(log_n_db=log_n_db, log_n_q=9, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9)
+    W = synth.make_workload(n_eyes=1, n_db=n_db, seed=21)
+    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    db = eng.encrypt_db(W.db_codes, W.db_masks)
+    s = eng.match(db, eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), 1, "f16_crt"))
+
+    def signed(codes, masks):      # +1 / -1 where the mask is set, else 0: sums below 2^24 are exact in fp32
+        c, m = (torch.as_tensor(np.asarray(x)).cuda().float() for x in (codes, masks))
+        return m - 2 * c * m
+
+    rc, rm = O.rotated_templates(W.q_codes, W.q_masks, eng.rho)
+    want = signed(rc, rm) @ signed(O.unpack(W.db_codes), O.unpack(W.db_masks)).T
+    assert torch.equal(eng.decrypt(s).cpu(), want.round().long().cpu())
