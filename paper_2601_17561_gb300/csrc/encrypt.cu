@@ -165,7 +165,7 @@ struct DbEncArgs {
     uint32_t K, eta, n_blocks, Lq, logc;             // 2^logc columns per block
     uint64_t seed, chunk;
     icm::NttMod nt[ICM_MAX_LIMBS];
-    const uint64_t *shat;                            // [blocks][L][N]: transforms of s_{db,t}, times N^-1
+    const ulonglong2 *shat;                          // [blocks][L][N]: transforms of s_{db,t}, times N^-1
     LimbTable lt;
     uint64_t *db;
 };
@@ -183,8 +183,8 @@ constexpr int NT_MUL = 512;
 // but a transform costs about 7 Shoup products per coefficient.  Columns are taken four at a time
 // where 2^14 words hold them, so that a row's words fill a 32-byte sector and the columns share
 // their twiddles.  1,000 templates at N_db = 2^12, four primes (4.0 GB): 69.5 ms with the
-// additions, 11.6 ms now (11 of them here: 6.6 the transforms, 2.3 the pointwise products, 1 the noise
-// and the rows' update, 0.8 drawing and storing the a-part).  Twice the threads (64 registers, the
+// additions, 10.95 ms now (10.3 of them here: 6.6 the transforms, 1.6 the pointwise products (2.3 without
+// the secrets' companions), 1 the noise and the rows' update, 0.8 drawing and storing the a-part).  Twice the threads (64 registers, the
 // polynomial kept in shared memory or not at all) or two blocks of half the columns give the same
 // time, one column per block 13.2 ms: multiplications bound it, not latency.
 template <int WPT>
@@ -218,12 +218,12 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant_
     }
     for (uint32_t t = 0; t < a.n_blocks; ++t) {
         // a thread overwrites only the words that it read itself
-        const uint64_t *sh = a.shat + ((size_t)t * a.lt.n + l) * N;
+        const ulonglong2 *sh = a.shat + ((size_t)t * a.lt.n + l) * N;
 #pragma unroll
         for (int j = 0; j < WPT; ++j) {
             const uint32_t x = threadIdx.x + j * NT_MUL;
             if (x < CN)
-                su[(x & (C - 1)) * stride + icm::ntt_pad(x >> a.logc)] = icm::mul_r128_lazy(ah[j], __ldg(sh + (x >> a.logc)), T);
+                su[(x & (C - 1)) * stride + icm::ntt_pad(x >> a.logc)] = icm::mul_lazy(ah[j], __ldg(sh + (x >> a.logc)), 0 - q);
         }
         __syncthreads();
         icm::ntt_inverse(su, C, stride, N, T);
@@ -251,7 +251,7 @@ struct QEncArgs {
     const uint8_t *codes, *masks;        // [n_eyes][code_bits/8]
     const uint64_t *eye_ids;
     icm::NttMod nt[2];
-    const uint64_t *shat;                // [nqblk][Lq][Nq]: transforms of s_{q,t}, times Nq^-1
+    const ulonglong2 *shat;              // [nqblk][Lq][Nq]: transforms of s_{q,t}, times Nq^-1
     uint64_t q[ICM_MAX_LIMBS], dl[ICM_MAX_LIMBS];   // primes and Delta mod q_l
     uint32_t n_cols;
     uint64_t *ct;                        // [Lq][n_cols][K]
@@ -259,7 +259,8 @@ struct QEncArgs {
 
 // One block per (2^logc query columns, limb l < Lq): the same transforms as k_db_apart_b.  32 eyes
 // (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient, 1.24 ms
-// with the column and eye of each word divided out, 1.01 ms now.
+// with the column and eye of each word divided out, 1.01 ms
+// with pointwise products by 128-bit reduction, 0.96 ms now.
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_constant__ QEncArgs a) {
     extern __shared__ uint64_t su[];                               // [2^logc][stride]
@@ -290,12 +291,12 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_consta
     }
     const uint32_t tb = a.code_bits / 8;
     for (uint32_t t = 0; t < a.nqblk; ++t) {
-        const uint64_t *sh = a.shat + ((size_t)t * a.Lq + l) * N;
+        const ulonglong2 *sh = a.shat + ((size_t)t * a.Lq + l) * N;
 #pragma unroll
         for (int w = 0; w < WPT; ++w) {
             const uint32_t x = threadIdx.x + w * NT_MUL;
             if (x < CN)
-                su[(x >> lgN) * stride + icm::ntt_pad(x & (N - 1))] = icm::mul_r128_lazy(ah[w], __ldg(sh + (x & (N - 1))), T);
+                su[(x >> lgN) * stride + icm::ntt_pad(x & (N - 1))] = icm::mul_lazy(ah[w], __ldg(sh + (x & (N - 1))), 0 - q);
         }
         __syncthreads();
         icm::ntt_inverse(su, C, stride, N, T);
@@ -339,6 +340,12 @@ __device__ __forceinline__ uint64_t mul_exact(uint64_t a, uint64_t b, const icm:
     const uint64_t r = icm::mul_r128_lazy(a, b, T);
     return r >= T.q ? r - T.q : r;
 }
+// (w, floor(w 2^64 / q)) for w < q: the estimate from floor(2^128 / q) is short by at most one
+__device__ __forceinline__ ulonglong2 with_companion(uint64_t w, const icm::NttMod &T) {
+    uint64_t ws = w * T.rhi + __umul64hi(w, T.rlo);
+    if ((uint64_t)0 - ws * T.q >= T.q) ++ws;
+    return make_ulonglong2(w, ws);
+}
 __global__ void k_ntt_table(const __grid_constant__ TabArgs a) {
     const uint32_t x = blockIdx.x * blockDim.x + threadIdx.x;
     if (x >= 2 * a.N) return;
@@ -346,10 +353,7 @@ __global__ void k_ntt_table(const __grid_constant__ TabArgs a) {
     uint64_t b = x >= a.N ? a.ipsi : a.psi, w = 1;
     for (; e; e >>= 1, b = mul_exact(b, b, a.T))
         if (e & 1) w = mul_exact(w, b, a.T);
-    // floor(w 2^64 / q): the estimate from floor(2^128 / q) is short by at most one
-    uint64_t ws = w * a.T.rhi + __umul64hi(w, a.T.rlo);
-    if ((uint64_t)0 - ws * a.T.q >= a.T.q) ++ws;
-    a.out[x] = make_ulonglong2(w, ws);
+    a.out[x] = with_companion(w, a.T);
 }
 
 // Transforms of the sparse secrets, times N^-1: one block per (secret t, limb l).
@@ -357,7 +361,7 @@ struct SecArgs {
     uint32_t N, h, L;
     icm::NttMod nt[ICM_MAX_LIMBS];
     const int32_t *pos; const int8_t *sgn;           // [t][h]
-    uint64_t *out;                                   // [t][L][N]
+    ulonglong2 *out;                                 // [t][L][N] (value, Shoup companion)
 };
 __global__ void __launch_bounds__(NT_MUL, 1) k_ntt_secret(const __grid_constant__ SecArgs a) {
     extern __shared__ uint64_t su[];
@@ -370,7 +374,7 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_ntt_secret(const __grid_constant_
     __syncthreads();
     icm::ntt_forward(su, 1, 0, a.N, T);
     for (uint32_t i = threadIdx.x; i < a.N; i += NT_MUL)
-        a.out[((size_t)t * a.L + l) * a.N + i] = mulmod_shoup(su[icm::ntt_pad(i)], T.ninv, T.ninvs, T.q);
+        a.out[((size_t)t * a.L + l) * a.N + i] = with_companion(mulmod_shoup(su[icm::ntt_pad(i)], T.ninv, T.ninvs, T.q), T);
 }
 
 }  // namespace
@@ -470,7 +474,7 @@ cudaError_t build_ntt(icm_ctx *c, std::string &why) {
         uint32_t logN = 0;
         while ((1u << logN) < N) ++logN;
         ulonglong2 **tab = w ? &S.tab_q : &S.tab_db;
-        uint64_t **shat = w ? &S.shat_q : &S.shat_db;
+        ulonglong2 **shat = w ? &S.shat_q : &S.shat_db;
         NttMod *nt = w ? S.q : S.db;
         cudaError_t e = cudaMalloc(tab, (size_t)L * 2 * N * sizeof(ulonglong2));
         if (e != cudaSuccess) return e;
@@ -490,7 +494,7 @@ cudaError_t build_ntt(icm_ctx *c, std::string &why) {
             TabArgs a{N, logN, psi, pow_mod(psi, q - 2, q), m, *tab + (size_t)l * 2 * N};
             k_ntt_table<<<(2 * N + 255) / 256, 256>>>(a);
         }
-        e = cudaMalloc(shat, (size_t)secrets[w] * L * N * 8);
+        e = cudaMalloc(shat, (size_t)secrets[w] * L * N * sizeof(ulonglong2));
         if (e != cudaSuccess) return e;
         SecArgs a{};
         a.N = N; a.h = c->p.hamming_weight; a.L = L;

@@ -91,7 +91,7 @@ struct DecArgs {
     uint32_t L, n_cols, shat_L;
     icm::NttMod nt[ICM_MAX_LIMBS];
     icm::CrtDecode crt;
-    const uint64_t *shat;  // [blocks][shat_L][N]: transforms of s_{db,t}, times N^-1
+    const ulonglong2 *shat;  // [blocks][shat_L][N]: transforms of s_{db,t}, times N^-1, with their companions
     const uint64_t *sc;    // [L][n_cols][M]
     int64_t *num;          // [n_cols][n_real]
     uint32_t *err_bits;    // optional: max |x - round(x)| over all outputs, as fp32 bits
@@ -115,7 +115,7 @@ __device__ __forceinline__ uint64_t ld_cluster(uint32_t addr, uint32_t rank) {
 // combines the limbs of each coefficient through distributed shared memory, so no limb goes through
 // global memory.  Integer products bound it (about 8 per coefficient and limb; the direct form added
 // h = 512 terms per coefficient, from L2).  8 eyes x 3,000 codes, 8 limbs, N_db = 2^12: 4.30 ms with
-// the direct form, 0.40 ms with one block of 512 threads per SM, 0.21 ms now.
+// the direct form, 0.40 ms with one block of 512 threads per SM, 0.20 ms now.
 template <int WPT, int NT, int MB>
 __global__ void __launch_bounds__(NT, MB) k_decrypt(const __grid_constant__ DecArgs a) {
     extern __shared__ uint64_t su[];
@@ -135,16 +135,16 @@ __global__ void __launch_bounds__(NT, MB) k_decrypt(const __grid_constant__ DecA
     }
     const uint32_t blocks = (uint32_t)((a.lay.n_real + N - 1) / N);
     for (uint32_t t = 0; t < blocks; ++t) {
-        const uint64_t *sh = a.shat + ((size_t)t * a.shat_L + l) * N;
+        const ulonglong2 *sh = a.shat + ((size_t)t * a.shat_L + l) * N;
         if (WPT == 0)
             for (uint32_t i = threadIdx.x; i < N; i += NT) {
                 uint64_t *w = su + icm::ntt_pad(i);
-                *w = icm::mul_r128_lazy(*w, __ldg(sh + i), T);
+                *w = icm::mul_lazy(*w, __ldg(sh + i), 0 - q);
             }
 #pragma unroll
         for (int w = 0; w < WPT; ++w) {
             const uint32_t i = threadIdx.x + w * NT;
-            if (i < N) su[icm::ntt_pad(i)] = icm::mul_r128_lazy(ah[w], __ldg(sh + i), T);
+            if (i < N) su[icm::ntt_pad(i)] = icm::mul_lazy(ah[w], __ldg(sh + i), 0 - q);
         }
         __syncthreads();
         icm::ntt_inverse(su, 1, 0, N, T);

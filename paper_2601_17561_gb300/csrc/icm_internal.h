@@ -45,7 +45,7 @@ struct RescaleConsts {
 struct NttSet {
     NttMod db[ICM_MAX_LIMBS] = {}, q[2] = {};
     ulonglong2 *tab_db = nullptr, *tab_q = nullptr;
-    uint64_t *shat_db = nullptr, *shat_q = nullptr;
+    ulonglong2 *shat_db = nullptr, *shat_q = nullptr;
     void release();
 };
 
