@@ -183,10 +183,11 @@ constexpr int NT_MUL = 512;
 // but a transform costs about 7 Shoup products per coefficient.  Columns are taken four at a time
 // where 2^14 words hold them, so that a row's words fill a 32-byte sector and the columns share
 // their twiddles.  1,000 templates at N_db = 2^12, four primes (4.0 GB): 69.5 ms with the
-// additions, 10.95 ms now (10.3 of them here: 6.6 the transforms, 1.6 the pointwise products (2.3 without
-// the secrets' companions), 1 the noise and the rows' update, 0.8 drawing and storing the a-part).  Twice the threads (64 registers, the
-// polynomial kept in shared memory or not at all) or two blocks of half the columns give the same
-// time, one column per block 13.2 ms: multiplications bound it, not latency.
+// additions, 10.95 ms now (10.3 of them here: 6.6 the transforms, 1.6 the pointwise products (2.3
+// without the secrets' companions), 1 the noise and the rows' update, 0.8 drawing and storing the
+// a-part).  Twice the threads (64 registers, the polynomial kept in shared memory or not at all) or
+// two blocks of half the columns give the same time, one column per block takes 13.2 ms:
+// multiplications bound it, not latency.
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant__ DbEncArgs a) {
     extern __shared__ uint64_t su[];                                     // [2^logc][stride]
@@ -258,9 +259,9 @@ struct QEncArgs {
 };
 
 // One block per (2^logc query columns, limb l < Lq): the same transforms as k_db_apart_b.  32 eyes
-// (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient, 1.24 ms
-// with the column and eye of each word divided out, 1.01 ms
-// with pointwise products by 128-bit reduction, 0.96 ms now.
+// (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient, 1.24 ms with
+// the column and eye of each word divided out, 1.01 ms with pointwise products by 128-bit reduction,
+// 0.96 ms now.
 template <int WPT>
 __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_constant__ QEncArgs a) {
     extern __shared__ uint64_t su[];                               // [2^logc][stride]
