@@ -21,11 +21,11 @@
 //   issues inside a lane-dependent branch and 40 on a successful barrier probe, beside the
 //   converters' issue slots; copies of 4 to 16 KB took it ~383 cycles each, so one copy per 16-deep
 //   slab and producer cannot feed a 256-cycle slab, while L2 itself delivers 117 B/clk/SM to several
-//   threads.  Here an operand stage is 32 deep (one copy of up to 32 KB per modulus), 
+//   threads.  Here an operand stage is 32 deep (one copy of up to 32 KB per modulus)
 //   and producers and issuer run on warp-uniform values with one elected lane.
 //   The MMA runs at 71 cycles for M 256 N 128 K 16 (64 is the peak; N 256 reaches 128 of 128, but
 //   needs twice the conversions): 570 cycles per 32-deep stage.
-//   Measured (GB300): 32 eyes against N_db + 16,384 rows, 8 limbs: 218 -> 168 ms per pass; 734 cycles
+//   Measured (GB300): 32 eyes against N_db + 16,384 rows, 8 limbs: 218 -> 161 to 166 ms per pass; 734 cycles
 //   per stage at the 1.75 GHz that the power limit leaves.  What is left is the ring: 4 stages of
 //   36 KB, of which an accumulator under reduction holds up to two.  Tried on this form: an issuer
 //   thread per accumulator (four commits per stage: 26 ms where this takes 19.4), two issuers
