@@ -41,7 +41,6 @@ DTYPE = {"u64": "u64", "i8_digits": "int8", "i8_crt": "int8", "f16_crt": "f16"}
 # figure scales one 512-column round by 2 rounds.  Absent (null) for a kernel changed since.
 NCU_TRAFFIC = {
     ("i8_crt", 0): 2 * 64 * (12_100_983_040 + 155_742_464),
-    ("u64", 0): 64 * (96_624_647_000 + 141_553_920),
 }
 
 
@@ -602,7 +601,8 @@ def main():
     h_ct = torch.empty(ct_bytes, dtype=torch.uint8, pin_memory=True)
     h_ct.copy_(ct[:ct_bytes].cpu())
     h_fo = torch.empty(fo_bytes, dtype=torch.uint8, pin_memory=True)
-    wsb = C.icm_match_host_workspace_bytes(eng.ctx, db.handle, N_EYES, f)
+    # workspace for all the eyes in one part (their columns share a round of the tcgen05 kernel)
+    wsb = C.icm_match_host_workspace_bytes(eng.ctx, db.handle, 2 * N_EYES, f)
     wsbuf = E._u8(wsb, dev)
     with torch.cuda.stream(st):
         C.icm_match_host(eng.ctx, db.handle, h_ct, N_EYES, f, h_fo, wsbuf, wsb, stream=st)
@@ -628,7 +628,7 @@ def main():
         """Roofline of the CCMM kernel of `form` from its CUDA-event time per launch."""
         tc = form == "f16_crt" and variant in (1, 2, 3)
         if form == "u64":
-            ops = 4.0 * M * n_cols * K * L                 # IMAD.WIDE per launch (2 x 2 30-bit limb products)
+            ops = 3.0 * M * n_cols * K * L                 # IMAD.WIDE per launch (three products of 30-bit halves)
             sm_max = peaks.get("sm_max_mhz", 2070.0)
             peak = 152 * 32 * sm_max * 1e6                  # 152 SMs x 32 IMAD.WIDE/clk x max SM clock
             roof = {"bound": "alu", "achieved": ops / gemm_avg_s / 1e9, "peak": peak / 1e9, "unit": "Gop/s",

@@ -393,7 +393,8 @@ icm_status icm_match_host_workspace_bytes(const icm_ctx *ctx, const icm_db *db, 
  * and joins back into `stream` (when `stream` completes, so has all of the call's work).  Host
  * buffers should be page-locked for asynchronous copies; they must stay valid until the stream
  * reaches the end of this work.  dev_ws: icm_match_host_workspace_bytes bytes of caller device
- * memory.  Errors: ICM_EINVAL (null arguments, no eyes), ICM_ENOMEM (workspace too small), and
+ * memory.  With the tcgen05 kernel two parts of up to 1,024 columns together convert the database
+ * twice; given the workspace of 2 n_eyes eyes, the call then runs them as one part.  Errors: ICM_EINVAL (null arguments, no eyes), ICM_ENOMEM (workspace too small), and
  * those of icm_query_prepare, icm_match and icm_fold. */
 icm_status icm_match_host(icm_ctx *ctx, const icm_db *db, const uint64_t *host_ct, size_t n_eyes, icm_form form,
                           uint64_t *host_folded, void *dev_ws, size_t ws_bytes, void *stream);

@@ -113,3 +113,21 @@ def test_ppmm_canonical(M, N, K):
     shifted.copy_(A)
     assert shifted.data_ptr() % 16 == 8
     assert torch.equal(E.ppmm("f16_crt", q, shifted, Bm), want)
+
+
+@pytest.mark.parametrize("n_eyes", [2, 8, 33, 34])
+def test_match_host_in_one_part(setup, n_eyes):
+    """icm_match_host with the workspace of twice the eyes (one part, where the columns share a round;
+    34 eyes need two and stay in two parts) gives the same folded residues as with its own."""
+    eng, W, dbs = setup
+    h_ct = eng.encrypt_query(W.q_codes[:n_eyes], W.q_masks[:n_eyes], W.eye_ids[:n_eyes]).cpu().pin_memory()
+    f, db, got = C.FORMS["f16_crt"], dbs[1], []
+    for n in (n_eyes, 2 * n_eyes):
+        wsb = C.icm_match_host_workspace_bytes(eng.ctx, db.handle, n, f)
+        ws = torch.empty(wsb, dtype=torch.uint8, device=eng.device)
+        h_fo = torch.zeros(eng.scores_bytes(db, n_eyes, True), dtype=torch.uint8).pin_memory()
+        st = torch.cuda.Stream()
+        C.icm_match_host(eng.ctx, db.handle, h_ct, n_eyes, f, h_fo, ws, wsb, stream=st)
+        st.synchronize()
+        got.append(h_fo)
+    assert got[0].any() and torch.equal(got[0], got[1])
