@@ -288,7 +288,8 @@ struct FwdArgs {
     const uint64_t *src; uint64_t src_ls, src_ps;
     uint64_t *dst; uint64_t dst_ls, dst_ps;
 };
-__global__ void __launch_bounds__(512, 2) k_ntt_fwd(const __grid_constant__ FwdArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_ntt_fwd(const __grid_constant__ FwdArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t total = (uint64_t)a.Lq * a.per_limb;
     for (uint64_t x = blockIdx.x; x < total; x += gridDim.x) {
@@ -310,7 +311,8 @@ __global__ void __launch_bounds__(512, 2) k_ntt_fwd(const __grid_constant__ FwdA
 // a_ntt holds NTT(a_j), mu_ntt NTT(mu_{j,t}); b rows are read from the rescaled scores.  The
 // transforms' integer products bound it; with three levels per pass over shared memory (ntt.cuh) and two
 // blocks per SM (64 registers) the normalisation of 8 eyes x 4,096 templates (N_db = 2^13) takes 652 us,
-// 738 us with one block, 820 us with one level per pass.
+// 738 us with one block, 820 us with one level per pass.  At N_db = 2^14, where one block of 1,024
+// threads fits, 32 eyes x 2^15 templates: 21.7 ms, 22.4 with 512 threads.
 struct MulArgs {
     icm::NttMod nt[2];
     uint32_t N, Lq, n_cols, n_blocks;
@@ -320,7 +322,8 @@ struct MulArgs {
     const uint64_t *mu_ntt;         // [Lq][n_cols][n_blocks][N]
     uint64_t *out;                  // [Lq][n_cols][n_blocks][2][N]
 };
-__global__ void __launch_bounds__(512, 2) k_ntt_mul_inv(const __grid_constant__ MulArgs a) {
+template <int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT) k_ntt_mul_inv(const __grid_constant__ MulArgs a) {
     extern __shared__ uint64_t su[];
     const uint64_t per_limb = (uint64_t)a.n_cols * a.n_blocks * 2;
     const uint64_t total = (uint64_t)a.Lq * per_limb;
@@ -640,24 +643,28 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
     // 3. NTT of every mu (in place) and of every a-part
     if (!c->nt.tab_db) return sfail(ICM_EINVAL, "icm_keygen has not run");
     const size_t psm = (size_t)ntt_words(N) * 8;
-    SL_TRY(set_smem(k_ntt_fwd, psm));
-    SL_TRY(set_smem(k_ntt_mul_inv, psm));
     // one polynomial per block in shared memory, as many blocks per SM as fit
     const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(4, (size_t)220 * 1024 / psm));
+    // 64 registers allow 1,024 threads per SM: two blocks, or one larger where only one polynomial fits
+    const unsigned ntt_threads = per_sm > 1 ? 512 : 1024;
+    auto *const fwd = per_sm > 1 ? k_ntt_fwd<512> : k_ntt_fwd<1024>;
+    auto *const mul_inv = per_sm > 1 ? k_ntt_mul_inv<512> : k_ntt_mul_inv<1024>;
+    SL_TRY(set_smem(fwd, psm));
+    SL_TRY(set_smem(mul_inv, psm));
     {
         FwdArgs a{};
         for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];
         a.N = N; a.Lq = Lq; a.per_limb = d3 * nb;
         a.src = mu; a.src_ls = (uint64_t)d3 * nb * N; a.src_ps = N;
         a.dst = mu; a.dst_ls = a.src_ls; a.dst_ps = N;
-        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * per_sm), 512, psm, st>>>(a);
+        fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(a);
         SL_TRY(cudaGetLastError());
         FwdArgs b{};
         for (uint32_t l = 0; l < Lq; ++l) b.nt[l] = c->nt.db[l];
         b.N = N; b.Lq = Lq; b.per_limb = d3;
         b.src = in->dev; b.src_ls = (uint64_t)d3 * in->lay.M; b.src_ps = in->lay.M;
         b.dst = antt; b.dst_ls = (uint64_t)d3 * N; b.dst_ps = N;
-        k_ntt_fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3, (uint64_t)sms * per_sm), 512, psm, st>>>(b);
+        fwd<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(b);
         SL_TRY(cudaGetLastError());
     }
     // 4. products and inverse NTTs
@@ -666,7 +673,7 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
         for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];
         a.N = N; a.Lq = Lq; a.n_cols = d3; a.n_blocks = nb; a.M = in->lay.M;
         a.scores = in->dev; a.a_ntt = antt; a.mu_ntt = mu; a.out = (uint64_t *)dev_out;
-        k_ntt_mul_inv<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb * 2, (uint64_t)sms * per_sm), 512, psm, st>>>(a);
+        mul_inv<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb * 2, (uint64_t)sms * per_sm), ntt_threads, psm, st>>>(a);
         SL_TRY(cudaGetLastError());
     }
     return ICM_OK;
