@@ -327,6 +327,9 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_consta
                 ct[i] = v;
             }
         }
+        // Word c N + i is written by thread (c N + i) mod NT_MUL above and read by thread i mod NT_MUL here:
+        // the same one unless a column is shorter than the block.
+        if (N < NT_MUL) __syncthreads();
     }
 }
 

@@ -77,3 +77,19 @@ def test_decryption_large_rings(log_n_db, n_db):
     rc, rm = O.rotated_templates(W.q_codes, W.q_masks, eng.rho)
     want = signed(rc, rm) @ signed(O.unpack(W.db_codes), O.unpack(W.db_masks)).T
     assert torch.equal(eng.decrypt(s).cpu(), want.round().long().cpu())
+
+
+# two columns of one block shorter than the block's 512 threads (n_eyes * 31 * Lq >= 304), one and two query primes,
+# an odd column count among them
+@pytest.mark.parametrize("log_n_q,L,Lq,n_eyes", [(5, 2, 1, 12), (5, 4, 2, 6), (7, 2, 1, 11), (7, 4, 2, 12), (8, 2, 1, 12),
+                                                 (8, 4, 2, 5), (9, 4, 2, 12)])
+def test_query_encryption_two_short_columns(log_n_q, L, Lq, n_eyes):
+    B.build()
+    prm = dict(log_n_db=5, log_n_q=log_n_q, n_limbs=L, n_limbs_q=Lq, prime_bits=60, log2_delta=60 if Lq == 2 else 40,
+               seed=9)
+    P = O.Params(**prm, h=16)
+    W = synth.make_workload(n_eyes=n_eyes, n_db=1, seed=21)
+    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    ct = O.query_encrypt(P, W.q_codes, W.q_masks, W.eye_ids)
+    for _ in range(3):
+        assert np.array_equal(_u64(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), ct.shape), ct)
