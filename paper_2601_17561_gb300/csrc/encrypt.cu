@@ -465,13 +465,13 @@ cudaError_t launch_query_encrypt(const icm_ctx *c, const uint8_t *d_codes, const
                               : launch_mul(k_query_encrypt<8>, a, grid, smem, st);
 }
 
-// Builds the transform tables and the secrets' transforms (icm_keygen, after the supports are on the
-// device).  Rings above 2^14 have no secret-product kernels and get no tables.
-cudaError_t build_ntt(icm_ctx *c, std::string &why) {
-    NttSet &S = c->nt;
-    S.release();
+// Builds the transform tables and the secrets' transforms into the empty set S (icm_keygen, from the supports
+// on the device; after an error the caller releases S).  Rings above 2^14 have no secret-product
+// kernels and get no tables.
+cudaError_t build_ntt(const icm_ctx *c, const int32_t *sdb_pos, const int8_t *sdb_sgn, uint32_t n_sdb, const int32_t *sq_pos,
+                      const int8_t *sq_sgn, NttSet &S, std::string &why) {
     const uint32_t rings[2] = {c->N_db, c->N_q}, limbs[2] = {c->p.n_limbs, c->p.n_limbs_q};
-    const uint32_t secrets[2] = {c->max_db_blocks, c->n_qblk};
+    const uint32_t secrets[2] = {n_sdb, c->n_qblk};
     for (int w = 0; w < 2; ++w) {
         const uint32_t N = rings[w], L = limbs[w];
         if (N > 16384) continue;
@@ -503,7 +503,7 @@ cudaError_t build_ntt(icm_ctx *c, std::string &why) {
         SecArgs a{};
         a.N = N; a.h = c->p.hamming_weight; a.L = L;
         for (uint32_t l = 0; l < L; ++l) a.nt[l] = nt[l];
-        a.pos = w ? c->d_sq_pos : c->d_sdb_pos; a.sgn = w ? c->d_sq_sgn : c->d_sdb_sgn;
+        a.pos = w ? sq_pos : sdb_pos; a.sgn = w ? sq_sgn : sdb_sgn;
         a.out = *shat;
         e = launch_mul(k_ntt_secret, a, dim3(secrets[w], L), (size_t)ntt_words(N) * 8, nullptr);
         if (e != cudaSuccess) return e;

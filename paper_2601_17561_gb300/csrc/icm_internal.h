@@ -149,7 +149,8 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
 // Rescaling by Q' of n coefficients per limb: [L][n] at modulus Q_db -> [L_q][n] at modulus Q.
 cudaError_t launch_rescale(const icm_ctx *c, const uint64_t *d_in, uint64_t n, uint64_t *d_out, cudaStream_t st);
 
-cudaError_t build_ntt(icm_ctx *c, std::string &why);
+cudaError_t build_ntt(const icm_ctx *c, const int32_t *sdb_pos, const int8_t *sdb_sgn, uint32_t n_sdb, const int32_t *sq_pos,
+                      const int8_t *sq_sgn, NttSet &S, std::string &why);
 uint64_t pow_mod(uint64_t b, uint64_t e, uint64_t q);
 cudaError_t launch_ppmm_cols(const icm_query *q, int bn, const I8Consts &k, ChunkTab &tab, const void *planes, uint64_t K,
                              void *scratch, cudaStream_t st);

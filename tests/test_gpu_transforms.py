@@ -93,3 +93,30 @@ def test_query_encryption_two_short_columns(log_n_q, L, Lq, n_eyes):
     ct = O.query_encrypt(P, W.q_codes, W.q_masks, W.eye_ids)
     for _ in range(3):
         assert np.array_equal(_u64(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), ct.shape), ct)
+
+
+def test_graphs_outlive_a_second_keygen():
+    """Decryption and normalisation captured before icm_keygen is called again replay on the transform tables that
+    they were captured with."""
+    B.build()
+    prm = dict(log_n_db=9, log_n_q=9, n_limbs=4, n_limbs_q=2, prime_bits=60, log2_delta=60, seed=9)
+    W = synth.make_workload(n_eyes=1, n_db=300, seed=21)
+    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    db, sdb = eng.encrypt_db(W.db_codes, W.db_masks), eng.encrypt_db_slots(W.db_codes, W.db_masks)
+    q = eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), 1, "u64")
+    s, r = eng.match(db, q), eng.rescale(eng.match(sdb, q))
+    qm, dm = torch.as_tensor(W.q_masks).cuda(), torch.as_tensor(W.db_masks).cuda()
+    nbytes, wbytes = E.C.icm_normalize_bytes(r.handle)
+    ws = torch.empty(wbytes, dtype=torch.uint8, device="cuda")
+    want = eng.decrypt(s), eng.normalize(r, qm, dm, ws=ws)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        got = eng.decrypt(s), eng.normalize(r, qm, dm, ws=ws)
+    eng.keygen()
+    E.Engine(**{**prm, "seed": 10}, hamming_weight=16).keygen()      # takes what the call above may have given back
+    for t in got:
+        t.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(got, want):
+        assert b.any() and torch.equal(a, b)
