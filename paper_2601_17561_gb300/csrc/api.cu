@@ -303,6 +303,14 @@ icm_status icm_keygen(icm_ctx *c) {
         cudaFree(a); cudaFree(b); cudaFree(x); cudaFree(y);
         return fail(ICM_ECUDA, std::string("keygen upload: ") + cudaGetErrorString(e));
     }
+    // shared-memory opt-ins are set here, outside any stream capture
+    e = encrypt_set_attributes();
+    if (e == cudaSuccess) e = decrypt_set_attributes();
+    if (e == cudaSuccess) e = slots_set_attributes();
+    if (e != cudaSuccess) {
+        cudaFree(a); cudaFree(b); cudaFree(x); cudaFree(y);
+        return fail(ICM_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
+    }
     // The transforms depend on the parameters alone (the secrets are drawn from the seed): a further call on
     // the same device keeps them where captured graphs read them, and a call that fails leaves the keys as
     // they were.
@@ -323,7 +331,6 @@ icm_status icm_keygen(icm_ctx *c) {
     c->max_db_blocks = max_blocks;
     c->device = dev;
     c->have_keys = true;
-    // shared-memory opt-ins of the product kernels are set once here, outside any stream capture
     e = crt_set_attributes();
     if (e != cudaSuccess) return fail(ICM_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
     return ICM_OK;

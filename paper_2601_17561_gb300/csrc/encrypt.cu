@@ -385,6 +385,11 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_ntt_secret(const __grid_constant_
 
 namespace icm {
 
+cudaError_t encrypt_set_attributes() {
+    return allow_smem(k_db_messages<false>, k_db_messages<true>, k_db_apart_b<8>, k_db_apart_b<16>, k_db_apart_b<32>,
+                      k_query_encrypt<8>, k_query_encrypt<16>, k_query_encrypt<32>, k_ntt_secret);
+}
+
 cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uint8_t *d_codes,
                                const uint8_t *d_masks, uint64_t *d_db, cudaStream_t st, const int32_t *d_wmsg) {
     DbMsgArgs a{};
@@ -401,8 +406,6 @@ cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uin
     const bool bits = !d_wmsg && (uint64_t)a.nqblk * a.h < 32768;
     const size_t smem = (bits ? (size_t)a.nqblk * (3 * a.Nq + 4) : (size_t)((a.d2 + 3) & ~3u) * 4) + (size_t)a.nqblk * a.h * 5;
     auto run = [&](auto kern) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         kern<<<(unsigned)nb, 512, smem, st>>>(a);
         return cudaGetLastError();
     };
@@ -419,8 +422,6 @@ static size_t mul_smem(uint32_t N, uint32_t logc) { return ((size_t)(ntt_words(N
 
 template <typename K, typename A>
 static cudaError_t launch_mul(K kern, const A &a, dim3 grid, size_t smem, cudaStream_t st) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     kern<<<grid, NT_MUL, smem, st>>>(a);
     return cudaGetLastError();
 }

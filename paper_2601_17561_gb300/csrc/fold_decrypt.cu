@@ -272,6 +272,11 @@ cudaError_t launch_fold(const icm_ctx *c, const LayoutDev &lay, const uint64_t *
     return cudaGetLastError();
 }
 
+cudaError_t decrypt_set_attributes() {
+    return allow_smem(k_decrypt<0, 256, 4>, k_decrypt<0, 512, 2>, k_decrypt<0, 1024, 1>, k_decrypt<16, 256, 3>,
+                      k_decrypt<32, 256, 2>, k_decrypt<16, 1024, 1>);
+}
+
 cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_t *d_scores, uint32_t n_cols,
                            bool rescaled, int64_t *d_num, cudaStream_t st, uint32_t *d_err_bits) {
     DecArgs a{};
@@ -285,8 +290,6 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
     if (!a.shat) return cudaErrorInvalidValue;                           // rings above 2^14
     const size_t smem = (size_t)ntt_words(lay.N) * 8;
     auto run = [&](auto kern, int nt) {
-        cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
         cudaLaunchConfig_t cfg = {};
         cudaLaunchAttribute attr[1];
         cfg.gridDim = dim3(a.L, n_cols); cfg.blockDim = dim3(nt);

@@ -149,6 +149,29 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
 // Rescaling by Q' of n coefficients per limb: [L][n] at modulus Q_db -> [L_q][n] at modulus Q.
 cudaError_t launch_rescale(const icm_ctx *c, const uint64_t *d_in, uint64_t n, uint64_t *d_out, cudaStream_t st);
 
+// Lets a kernel be launched with all the shared memory that a block can have.  Set once per device
+// (icm_keygen): a limit set before each launch to that launch's size could be lowered by another host
+// thread, with a smaller ring, before the launch.
+template <typename K>
+cudaError_t allow_smem(K kern) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, kern);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, optin - (int)fa.sharedSizeBytes);
+    return e;
+}
+template <typename K, typename... R>
+cudaError_t allow_smem(K kern, R... rest) {
+    const cudaError_t e = allow_smem(kern);
+    return e != cudaSuccess ? e : allow_smem(rest...);
+}
+cudaError_t encrypt_set_attributes();
+cudaError_t decrypt_set_attributes();
+cudaError_t slots_set_attributes();
+
 cudaError_t build_ntt(const icm_ctx *c, const int32_t *sdb_pos, const int8_t *sdb_sgn, uint32_t n_sdb, const int32_t *sq_pos,
                       const int8_t *sq_sgn, NttSet &S, std::string &why);
 uint64_t pow_mod(uint64_t b, uint64_t e, uint64_t q);

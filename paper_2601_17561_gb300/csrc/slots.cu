@@ -452,12 +452,12 @@ int sm_count() {
     return sms > 0 ? sms : 1;
 }
 
-template <typename K>
-cudaError_t set_smem(K kern, size_t bytes) {
-    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-}
-
 }  // namespace
+
+cudaError_t slots_set_attributes() {
+    return allow_smem(k_slot_db_encode, k_mu_encode, k_ntt_fwd<512>, k_ntt_fwd<1024>, k_ntt_mul_inv<512>,
+                      k_ntt_mul_inv<1024>, k_slot_dec_limbs, k_slot_decode);
+}
 
 // Workspace layout of icm_normalize (offsets 256-byte aligned): rotated query masks [n_cols][1600],
 // mask overlaps [n_cols][n_tpl] int32, mu residues [Lq][n_cols][n_blocks][N], NTT(a) [Lq][n_cols][N].
@@ -554,13 +554,10 @@ icm_status icm_db_encrypt_slots(icm_ctx *c, const uint8_t *codes, const uint8_t 
         a.scale = ldexp(1.0, (int)log2_scale);
         a.twist = T->twist; a.tw = T->tw; a.pos = T->pos; a.W = d_w;
         const size_t smem = (size_t)n * 16 + (size_t)(n / 2) * 16;
-        e = set_smem(k_slot_db_encode, smem);
-        if (e == cudaSuccess) {
-            const uint64_t total = nb * c->p.code_bits;
-            const unsigned grid = (unsigned)std::min<uint64_t>(total, (uint64_t)sm_count() * (smem > 110000 ? 1 : 2));
-            k_slot_db_encode<<<grid, 512, smem, st>>>(a);
-            e = cudaGetLastError();
-        }
+        const uint64_t total = nb * c->p.code_bits;
+        const unsigned grid = (unsigned)std::min<uint64_t>(total, (uint64_t)sm_count() * (smem > 110000 ? 1 : 2));
+        k_slot_db_encode<<<grid, 512, smem, st>>>(a);
+        e = cudaGetLastError();
     }
     icm_db *db = nullptr;
     if (e == cudaSuccess) {
@@ -635,7 +632,6 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
         for (uint32_t l = 0; l < Lq; ++l) a.q[l] = c->q[l];
         a.mu = mu;
         const size_t smem = (size_t)n * 16 + (size_t)(n / 2) * 16;
-        SL_TRY(set_smem(k_mu_encode, smem));
         const unsigned grid = (unsigned)std::min<uint64_t>((uint64_t)d3 * nb, (uint64_t)sms * (smem > 110000 ? 1 : 2));
         k_mu_encode<<<grid, 512, smem, st>>>(a);
         SL_TRY(cudaGetLastError());
@@ -649,8 +645,6 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
     const unsigned ntt_threads = per_sm > 1 ? 512 : 1024;
     auto *const fwd = per_sm > 1 ? k_ntt_fwd<512> : k_ntt_fwd<1024>;
     auto *const mul_inv = per_sm > 1 ? k_ntt_mul_inv<512> : k_ntt_mul_inv<1024>;
-    SL_TRY(set_smem(fwd, psm));
-    SL_TRY(set_smem(mul_inv, psm));
     {
         FwdArgs a{};
         for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];
@@ -704,11 +698,8 @@ icm_status icm_decrypt_slots(icm_ctx *c, const icm_scores *in, const void *dev_n
         a.spos = c->d_sdb_pos; a.ssgn = c->d_sdb_sgn;
         a.norm = (const uint64_t *)dev_norm; a.dec = dec;
         const size_t psm = (size_t)N * 8;
-        e = set_smem(k_slot_dec_limbs, psm);
-        if (e == cudaSuccess) {
-            k_slot_dec_limbs<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * 2), 512, psm, st>>>(a);
-            e = cudaGetLastError();
-        }
+        k_slot_dec_limbs<<<(unsigned)std::min<uint64_t>((uint64_t)Lq * d3 * nb, (uint64_t)sms * 2), 512, psm, st>>>(a);
+        e = cudaGetLastError();
     }
     if (e == cudaSuccess) {
         DecodeArgs a{};
@@ -718,12 +709,9 @@ icm_status icm_decrypt_slots(icm_ctx *c, const icm_scores *in, const void *dev_n
         a.inv_scale = ldexp(1.0, -(int)(c->p.log2_delta + in->lay.slot_log2 + log2_scale_mu));
         a.twist = T->twist; a.tw = T->tw; a.pos = T->pos; a.dec = dec; a.hd = dev_hd;
         const size_t smem = (size_t)n2 * 16 + (size_t)(n2 / 2) * 16;
-        e = set_smem(k_slot_decode, smem);
-        if (e == cudaSuccess) {
-            k_slot_decode<<<(unsigned)std::min<uint64_t>((uint64_t)d3 * nb, (uint64_t)sms * (smem > 110000 ? 1 : 2)),
-                            512, smem, st>>>(a);
-            e = cudaGetLastError();
-        }
+        k_slot_decode<<<(unsigned)std::min<uint64_t>((uint64_t)d3 * nb, (uint64_t)sms * (smem > 110000 ? 1 : 2)), 512,
+                        smem, st>>>(a);
+        e = cudaGetLastError();
     }
     cudaFreeAsync(dec, st);
     if (e != cudaSuccess) return sfail(ICM_ECUDA, std::string("slot decrypt: ") + cudaGetErrorString(e));

@@ -1,6 +1,8 @@
 """The encryption kernels' products by the secrets (negacyclic transforms) at the edges of their range: the
 smallest rings, one, two and four columns per block, partial blocks, two query primes, against the
 oracle bit by bit."""
+import threading
+
 import numpy as np
 import pytest
 import torch
@@ -120,3 +122,37 @@ def test_graphs_outlive_a_second_keygen():
     torch.cuda.synchronize()
     for a, b in zip(got, want):
         assert b.any() and torch.equal(a, b)
+
+
+def test_decryption_from_two_threads():
+    """Two contexts of different rings decrypt from two host threads: no launch meets the other one's limit of
+    dynamic shared memory."""
+    B.build()
+    work = []
+    for log_n_db in (5, 12):
+        eng = E.Engine(log_n_db=log_n_db, log_n_q=9, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9,
+                       hamming_weight=16).keygen()
+        W = synth.make_workload(n_eyes=1, n_db=20, seed=21)
+        s = eng.match(eng.encrypt_db(W.db_codes, W.db_masks),
+                      eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), 1, "u64"))
+        out = torch.zeros(31 * 20, dtype=torch.int64, device="cuda")
+        work.append((eng, s, out, eng.decrypt(s).flatten(), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    errors = []
+
+    def loop(eng, s, out, want, st):
+        try:
+            for _ in range(4000):
+                E.C.icm_decrypt_scores(eng.ctx, s.handle, out, out.numel(), stream=st)
+        except Exception as e:
+            errors.append(e)
+
+    threads = [threading.Thread(target=loop, args=w) for w in work]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    torch.cuda.synchronize()
+    assert not errors
+    for _, _, out, want, _ in work:
+        assert torch.equal(out, want)
