@@ -937,6 +937,11 @@ cudaError_t crt_tc_set_attributes() {
     return e;
 }
 
+// Deepest product of the digit form: the carries out of the top digit are summed in fp32.  An interval of 960
+// products adds at most 4,082 to the sum (top digits of weights below 2^59 in magnitude are at most 8:
+// (960 128 8 + 61,690) / 256), so the 2,185 intervals of 2^18 words stay below 2^24 (8.92e6); 493,200 words would too.
+constexpr uint64_t DIG_MAX_K = 1ull << 18;
+
 // The digit form takes the columns that would leave the last group of 256 nearly empty, where its planes
 // fit the residue planes' place in the operand (so that buffer sizes do not depend on the choice): up to
 // n_mod / 8 groups of 32 columns, 2 for 60-bit primes.  One pass of a row tile per group costs 2,048 cycles
@@ -946,7 +951,7 @@ cudaError_t crt_tc_set_attributes() {
 uint32_t dig_cols(uint32_t n_mod, uint64_t N, uint64_t K) {
     const uint32_t rem = (uint32_t)(N % 256), g = (rem + 31) / 32;
     const bool pays = g == 1 || (g == 2 && (N / 256) % 2 == 0);
-    return pays && g * 8 <= n_mod && crt_tc_supported(K) ? rem : 0;
+    return pays && g * 8 <= n_mod && crt_tc_supported(K) && K <= DIG_MAX_K ? rem : 0;
 }
 
 cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N, uint64_t K,

@@ -261,3 +261,23 @@ def test_p2_digit_split_exhaustive():
         assert np.all(np.abs(x0) <= h) and np.all(x0 + p * x1 == x), p
         worst = max(worst, int(np.abs(x1).max()))
     assert worst == 126
+
+
+def _dig_cols(lib, n_mod, n, k):
+    f = C.lib()["_ZN3icm8dig_colsEjmm"]
+    f.restype, f.argtypes = ctypes.c_uint32, [ctypes.c_uint32, ctypes.c_uint64, ctypes.c_uint64]
+    return f(n_mod, n, k)
+
+
+def test_digit_form_depth(lib):
+    """The digit form of the fp16 product sums the carries out of its top digit in fp32: wherever it is chosen, their
+    largest possible sum (every digit product at its extreme, weights below 2^59 in magnitude) is an exact float."""
+    def top_sum(k):
+        carry = 0                                           # largest carry into digit u of an interval of 960 products
+        for u in range(8):
+            digit = 128 if u < 7 else 8                     # |d_7| of a centred value below 2^59
+            carry = (960 * 128 * digit + 128 + carry + 128) // 256
+        return -(-2 * -(-k // 16) // 15) * carry
+    assert _dig_cols(lib, 18, 31, 24576) == 31
+    for k in (2, 24576, 1 << 18, (1 << 18) + 2, 1 << 19, 1 << 20, 1 << 24, (1 << 32) - 2):
+        assert not _dig_cols(lib, 18, 31, k) or top_sum(k) < 1 << 24, k
