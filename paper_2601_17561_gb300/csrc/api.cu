@@ -436,7 +436,7 @@ icm_status icm_query_prepare(icm_ctx *c, const void *dev_ct, size_t n_eyes, icm_
     if (e == cudaSuccess && form != ICM_FORM_U64) {
         const I8Consts &k = form == ICM_FORM_I8_DIGITS ? c->i8_digits : c->i8_crt;
         int8_t *planes = (int8_t *)dev_op + (size_t)c->p.n_limbs * n_cols * c->K * 8;
-        const uint32_t n_dig = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) ? dig_cols(k.n_mod, n_cols, c->K) : 0;
+        const uint32_t n_dig = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) ? dig_cols(k.n_mod, c->p.n_limbs, c->N_db, n_cols, c->K) : 0;
         q->n_crt = n_cols - n_dig;
         if (n_dig) {
             const uint64_t Kp = i8_kpad(c->K);
@@ -484,7 +484,7 @@ icm_status icm_match_launches(const icm_ctx *c, const icm_db *db, size_t n_eyes,
     if (form != ICM_FORM_I8_CRT && form != ICM_FORM_F16_CRT) return fail(ICM_EINVAL, "not a match form");
     const uint32_t L = c->p.n_limbs, G = crt_limb_group(L, c->i8_crt.n_mod, N, M);
     const bool tc = form == ICM_FORM_F16_CRT && crt_tc_variant(c->crt_bn) && crt_tc_supported(c->K);
-    const uint64_t cols = tc ? 1024 : 512, n_dig = tc ? dig_cols(c->i8_crt.n_mod, N, c->K) : 0;
+    const uint64_t cols = tc ? 1024 : 512, n_dig = tc ? dig_cols(c->i8_crt.n_mod, L, c->N_db, N, c->K) : 0;
     *n = (size_t)((L + G - 1) / G) * ((N - n_dig + cols - 1) / cols) * 2 + (n_dig ? 1 : 0);
     return ICM_OK;
 }

@@ -948,10 +948,15 @@ constexpr uint64_t DIG_MAX_K = 1ull << 18;
 // per 16 words and 256 rows whatever the rest.  Measured for 8,192 rows and 8 limbs (ms): digits 3.6 per
 // group; residues 13.2, 19.9, 33.4, 40.3 for one to four groups of 256.  So one group of 32 always
 // goes to the digits, two where the last group of 256 would be the first or third of its launch.
-uint32_t dig_cols(uint32_t n_mod, uint64_t N, uint64_t K) {
+// Past residue columns they take a further launch, one pass of K (0.85 ms at K = 20,480) whatever the rows, which
+// a database of few row tiles does not repay.  9 eyes against N_db + 630 rows (ms; all columns as residues on
+// mma.sync in brackets): N_db = 2^11 on two limbs 2.00 (1.82), on three 2.30 (2.93); 2^12 on two 2.58 (3.24);
+// 2^10 on two, as residues here, 1.14 (1.49).  A database has at least N_db rows.
+uint32_t dig_cols(uint32_t n_mod, uint32_t n_limbs, uint32_t n_db, uint64_t N, uint64_t K) {
     const uint32_t rem = (uint32_t)(N % 256), g = (rem + 31) / 32;
     const bool pays = g == 1 || (g == 2 && (N / 256) % 2 == 0);
-    return pays && g * 8 <= n_mod && crt_tc_supported(K) && K <= DIG_MAX_K ? rem : 0;
+    const bool rows = N < 256 || (uint64_t)n_limbs * n_db >= 6144;
+    return pays && rows && g * 8 <= n_mod && crt_tc_supported(K) && K <= DIG_MAX_K ? rem : 0;
 }
 
 cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N, uint64_t K,

@@ -69,10 +69,11 @@ cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const voi
 cudaError_t crt_tc_set_attributes();
 bool crt_tc_supported(uint64_t K);
 bool crt_tc_aligned(const ChunkTab &tab);
-// Digit form of the fp16 product (ppmm_dig_tc.cuh): how many of the last columns of N it takes (0: none);
+// Digit form of the fp16 product (ppmm_dig_tc.cuh): how many of the last columns of N it takes (0: none) on a
+// database of ring degree n_db;
 // its planes follow the residue planes of the others, within their place for N columns.  The planes are
 // made from n columns at `op` of an operand of n_op columns; the product writes columns col0 ...
-uint32_t dig_cols(uint32_t n_mod, uint64_t N, uint64_t K);
+uint32_t dig_cols(uint32_t n_mod, uint32_t n_limbs, uint32_t n_db, uint64_t N, uint64_t K);
 cudaError_t launch_dig_planes(const I8Consts &k, const uint64_t *op, uint64_t n_op, void *planes, uint64_t N, uint64_t K,
                               uint64_t Kp, cudaStream_t st);
 cudaError_t launch_ppmm_dig(const I8Consts &k, const ChunkTab &tab, const void *Bp, uint64_t col0, uint64_t N, uint64_t K,

@@ -131,3 +131,33 @@ def test_match_host_in_one_part(setup, n_eyes):
         st.synchronize()
         got.append(h_fo)
     assert got[0].any() and torch.equal(got[0], got[1])
+
+
+@pytest.fixture(scope="module")
+def rows():
+    # N_db = 2^11 on three limbs: the fewest rows beside which the last columns go to the digit planes
+    eng = E.Engine(log_n_db=11, log_n_q=5, n_limbs=3, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=8,
+                   hamming_weight=16).keygen()
+    W = synth.make_workload(n_eyes=40, n_db=300, seed=35)
+    return eng, W, [eng.encrypt_db(W.db_codes[a:b], W.db_masks[a:b], chunk_id=i) for i, (a, b) in enumerate([(0, 3), (3, 300)])]
+
+
+@pytest.mark.parametrize("n_eyes,launches", [(9, 3), (17, 3), (34, 3), (40, 4)])
+def test_digits_beside_residues(rows, n_eyes, launches):
+    """One, two and four groups of 256 columns as residues and the rest as digits (279, 527, 1,054 columns), and a
+    second round of residues (1,240 columns), on the storage form: the residues of the mma.sync kernel."""
+    eng, W, dbs = rows
+    assert C.icm_match_launches(eng.ctx, dbs[1].handle, n_eyes, C.FORMS["f16_crt"]) == launches
+    ct = eng.encrypt_query(W.q_codes[:n_eyes], W.q_masks[:n_eyes], W.eye_ids[:n_eyes])
+    res = []
+    try:
+        for v in (256, 2):
+            C.icm_ctx_set_variant(eng.ctx, v)
+            outs = eng.match_batch(dbs, eng.prepare(ct, n_eyes, "f16_crt"))
+            torch.cuda.synchronize()
+            res.append([s.residues() for s in outs])
+    finally:
+        C.icm_ctx_set_variant(eng.ctx, 0)
+    C.icm_device_status(True)
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)

@@ -263,10 +263,10 @@ def test_p2_digit_split_exhaustive():
     assert worst == 126
 
 
-def _dig_cols(lib, n_mod, n, k):
-    f = C.lib()["_ZN3icm8dig_colsEjmm"]
-    f.restype, f.argtypes = ctypes.c_uint32, [ctypes.c_uint32, ctypes.c_uint64, ctypes.c_uint64]
-    return f(n_mod, n, k)
+def _dig_cols(lib, n_mod, n, k, n_limbs=8, n_db=4096):
+    f = C.lib()["_ZN3icm8dig_colsEjjjmm"]
+    f.restype, f.argtypes = ctypes.c_uint32, [ctypes.c_uint32] * 3 + [ctypes.c_uint64] * 2
+    return f(n_mod, n_limbs, n_db, n, k)
 
 
 def test_digit_form_depth(lib):
@@ -281,3 +281,10 @@ def test_digit_form_depth(lib):
     assert _dig_cols(lib, 18, 31, 24576) == 31
     for k in (2, 24576, 1 << 18, (1 << 18) + 2, 1 << 19, 1 << 20, 1 << 24, (1 << 32) - 2):
         assert not _dig_cols(lib, 18, 31, k) or top_sum(k) < 1 << 24, k
+
+
+def test_digit_form_needs_rows_beside_residues(lib):
+    """Columns past a multiple of 256 go to a second launch only where the database fills it."""
+    for n_limbs, n_db, n, want in [(2, 1 << 7, 31, 31), (2, 1 << 10, 279, 0), (2, 1 << 11, 527, 0), (3, 1 << 11, 279, 23),
+                                   (2, 1 << 12, 279, 23), (8, 1 << 14, 992, 0), (3, 1 << 12, 527, 15)]:
+        assert _dig_cols(lib, 18, n, 20480, n_limbs, n_db) == want, (n_limbs, n_db, n)
