@@ -14,6 +14,7 @@
 //   where column j = eye * rho + r holds rotation r of the eye (Section 2.1.2).
 #include "icm_internal.h"
 
+#include <algorithm>
 #include <string>
 
 namespace {
@@ -166,6 +167,8 @@ struct DbEncArgs {
     uint64_t seed, chunk;
     icm::NttMod nt[ICM_MAX_LIMBS];
     const ulonglong2 *shat;                          // [blocks][L][N]: transforms of s_{db,t}, times N^-1
+    uint32_t h;
+    const int32_t *sdb_pos; const int8_t *sdb_sgn;   // [blocks][h]: the supports, for the direct form
     LimbTable lt;
     uint64_t *db;
 };
@@ -243,6 +246,47 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_db_apart_b(const __grid_constant_
             v = e >= 0 ? add_mod(v, (uint64_t)e, q) : sub_mod(v, (uint64_t)(-e), q);
             *dst = to_digit_form(v, q);
         }
+    }
+}
+
+// Pass 2 in the direct form, one block per (column k, limb l): h additions per stored b-row.  A chunk of few
+// templates stores few rows of its ring (and small rings leave most of a transform's threads idle):
+// db_direct says where that is the cheaper one.
+__global__ void __launch_bounds__(1024) k_db_apart_b_direct(const __grid_constant__ DbEncArgs a) {
+    extern __shared__ uint64_t su[];
+    uint64_t *acol = su;                                                 // [N]
+    int32_t *spos = reinterpret_cast<int32_t *>(acol + a.lay.N);         // [n_blocks * h]
+    int8_t *ssgn = reinterpret_cast<int8_t *>(spos + a.n_blocks * a.h);
+    const uint32_t k = blockIdx.x, l = blockIdx.y, N = a.lay.N;
+    const uint64_t q = a.lt.q[l];
+    const uint64_t ka = stream_key(a.seed, ICM_KIND_A_DB, a.chunk, l);
+    const uint64_t ke = stream_key(a.seed, ICM_KIND_E_DB, a.chunk, 0);
+    uint64_t *dbl = a.db + (size_t)l * a.lay.M * a.K;
+    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
+        const uint64_t v = uniform_mod(sm64(ka, (uint64_t)i * a.K + k), q);
+        acol[i] = v;
+        dbl[(size_t)i * a.K + k] = to_digit_form(v, q);
+    }
+    for (uint32_t x = threadIdx.x; x < a.n_blocks * a.h; x += blockDim.x) { spos[x] = a.sdb_pos[x]; ssgn[x] = a.sdb_sgn[x]; }
+    __syncthreads();
+    const uint64_t nb = a.lay.M - N;
+    for (uint64_t bidx = threadIdx.x; bidx < nb; bidx += blockDim.x) {
+        uint32_t t, i;
+        b_row_of(a.lay, bidx, t, i);
+        uint64_t sa = 0;                                                 // (s_{db,t} * a)[i] mod q
+        for (uint32_t c = 0; c < a.h; ++c) {
+            // X^p X^(i-p): wraps with a sign flip when i < p
+            const uint32_t p = (uint32_t)spos[t * a.h + c];
+            const int s = ssgn[t * a.h + c];
+            const uint64_t term = (i >= p) ? acol[i - p] : acol[N + i - p];
+            const bool neg = (i >= p) ? (s < 0) : (s > 0);
+            sa = neg ? sub_mod(sa, term, q) : add_mod(sa, term, q);
+        }
+        uint64_t *dst = dbl + (size_t)(N + bidx) * a.K + k;
+        const int e = cbd_sample(sm64(ke, ((uint64_t)t * N + i) * a.K + k), a.eta);
+        uint64_t v = sub_mod(l < a.Lq ? *dst : 0, sa, q);
+        v = e >= 0 ? add_mod(v, (uint64_t)e, q) : sub_mod(v, (uint64_t)(-e), q);
+        *dst = to_digit_form(v, q);
     }
 }
 
@@ -386,7 +430,7 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_ntt_secret(const __grid_constant_
 namespace icm {
 
 cudaError_t encrypt_set_attributes() {
-    return allow_smem(k_db_messages<false>, k_db_messages<true>, k_db_apart_b<8>, k_db_apart_b<16>, k_db_apart_b<32>,
+    return allow_smem(k_db_messages<false>, k_db_messages<true>, k_db_apart_b_direct, k_db_apart_b<8>, k_db_apart_b<16>, k_db_apart_b<32>,
                       k_query_encrypt<8>, k_query_encrypt<16>, k_query_encrypt<32>, k_ntt_secret);
 }
 
@@ -426,6 +470,17 @@ static cudaError_t launch_mul(K kern, const A &a, dim3 grid, size_t smem, cudaSt
     return cudaGetLastError();
 }
 
+// Whether h additions per stored b-row cost less than a forward transform and an inverse one per block, per
+// column and limb.  Measured in additions (1.24 ps each), a transform takes 7 per coefficient, and 4,500 in rings
+// below 2^9, which leave its threads idle.  L = 4, ms, additions / transforms:
+//   h = 512, 100 templates: N_db = 2^12 11.6 / 8.4, 2^13 16.0 / 22.3, 2^14 21.6 / 52.6
+//   h = 512, 1,000: 2^13 70.7 / 23.6;  h = 64, 3,000: 2^7 18.7 / 18.7, 2^8 18.5 / 10.8, 2^12 23.4 / 10.6
+//   h = 64, 100: 2^12 3.8 / 8.3, 2^11 2.5 / 4.0, 2^10 2.3 / 2.3;  h = 16, 3,000: 2^5 8.5 / 39.8, 2^7 7.3 / 14.6
+static bool db_direct(uint32_t h, uint32_t N, uint32_t n_blocks, uint64_t rows) {
+    return rows * h < (uint64_t)(n_blocks + 1) * std::max(7 * N, 4500u) &&
+           (size_t)N * 8 + (size_t)n_blocks * h * 5 <= 200 * 1024;
+}
+
 cudaError_t launch_db_apart_and_b(const icm_ctx *c, const LayoutDev &lay, uint64_t chunk_id, uint64_t *d_db,
                                   cudaStream_t st) {
     if (!c->nt.shat_db) return cudaErrorInvalidValue;                    // rings above 2^14
@@ -437,6 +492,12 @@ cudaError_t launch_db_apart_and_b(const icm_ctx *c, const LayoutDev &lay, uint64
     for (uint32_t l = 0; l < c->p.n_limbs; ++l) a.nt[l] = c->nt.db[l];
     a.shat = c->nt.shat_db;
     a.lt = c->lt; a.db = d_db;
+    if (db_direct(c->p.hamming_weight, lay.N, a.n_blocks, lay.M - lay.N)) {
+        a.h = c->p.hamming_weight; a.sdb_pos = c->d_sdb_pos; a.sdb_sgn = c->d_sdb_sgn;
+        const size_t smem = (size_t)lay.N * 8 + (size_t)a.n_blocks * a.h * 5;
+        k_db_apart_b_direct<<<dim3(c->K, c->p.n_limbs), 1024, smem, st>>>(a);
+        return cudaGetLastError();
+    }
     const size_t smem = mul_smem(lay.N, a.logc);
     dim3 grid((c->K + (1u << a.logc) - 1) >> a.logc, c->p.n_limbs);
     const uint32_t wpt = (uint32_t)(((uint64_t)lay.N << a.logc) + NT_MUL - 1) / NT_MUL;

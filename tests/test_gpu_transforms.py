@@ -156,3 +156,41 @@ def test_decryption_from_two_threads():
     assert not errors
     for _, _, out, want, _ in work:
         assert torch.equal(out, want)
+
+
+# chunks whose b-rows go through the transforms (h additions per row would cost more): four columns per block in
+# rings of 2^7 to 2^12, two in 2^13; several blocks, partial ones
+@pytest.mark.parametrize("log_n_db,h,n_db", [(7, 128, 300), (9, 512, 40), (10, 256, 1100), (11, 512, 90), (12, 512, 100),
+                                             (13, 2048, 40)])
+def test_database_encryption_by_transforms(log_n_db, h, n_db):
+    B.build()
+    prm = dict(log_n_db=log_n_db, log_n_q=max(7, (h - 1).bit_length()), n_limbs=2, n_limbs_q=1, prime_bits=60,
+               log2_delta=40, seed=9)
+    P = O.Params(**prm, h=h)
+    W = synth.make_workload(n_eyes=1, n_db=n_db, seed=21)
+    eng = E.Engine(**prm, hamming_weight=h).keygen()
+    A = O.db_rows(P, W.db_codes, W.db_masks, O.db_layout(n_db, P.ndb, P.rho))
+    db = eng.encrypt_db(W.db_codes, W.db_masks)
+    assert np.array_equal(_from_digit_form(_u64(db.buf, A.shape), P.q), A)
+
+
+def _best_ms(f):
+    t = []
+    for _ in range(4):
+        a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+        a.record()
+        f()
+        b.record()
+        torch.cuda.synchronize()
+        t.append(a.elapsed_time(b))
+    return min(t)
+
+
+def test_few_templates_in_a_large_ring():
+    """100 templates store 130 rows of a ring of 2^14: they add less to the 2^14 rows of the a-part than a
+    transform over the ring and back would (three times the a-part's own time)."""
+    B.build()
+    eng = E.Engine(log_n_db=14, log_n_q=9, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9).keygen()
+    W = synth.make_workload(n_eyes=1, n_db=100, seed=21)
+    empty = _best_ms(lambda: eng.encrypt_db(W.db_codes[:0], W.db_masks[:0]))
+    assert _best_ms(lambda: eng.encrypt_db(W.db_codes, W.db_masks)) < 2.5 * empty
