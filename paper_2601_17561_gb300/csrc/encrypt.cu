@@ -446,8 +446,10 @@ cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uin
     a.db = d_db;
     const uint64_t nb = lay.M - lay.N;
     if (nb == 0) return cudaSuccess;
-    // 16-bit sums of bytes below 3 hold 32,767 terms
-    const bool bits = !d_wmsg && (uint64_t)a.nqblk * a.h < 32768;
+    // 16-bit sums of bytes below 3 hold 32,767 terms.  A query ring below 2^10 has at most 128 words of four
+    // entries for 512 threads; one addition at a time then leaves fewer idle (3,000 templates, h = 512, two limbs
+    // of N_db = 2^12: N_q = 2^9 24.4 ms with words of four, 15.5 without; 2^10 10.9 and 15.1).
+    const bool bits = !d_wmsg && a.Nq >= 1024 && (uint64_t)a.nqblk * a.h < 32768;
     const size_t smem = (bits ? (size_t)a.nqblk * (3 * a.Nq + 4) : (size_t)((a.d2 + 3) & ~3u) * 4) + (size_t)a.nqblk * a.h * 5;
     auto run = [&](auto kern) {
         kern<<<(unsigned)nb, 512, smem, st>>>(a);

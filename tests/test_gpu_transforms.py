@@ -194,3 +194,15 @@ def test_few_templates_in_a_large_ring():
     W = synth.make_workload(n_eyes=1, n_db=100, seed=21)
     empty = _best_ms(lambda: eng.encrypt_db(W.db_codes[:0], W.db_masks[:0]))
     assert _best_ms(lambda: eng.encrypt_db(W.db_codes, W.db_masks)) < 2.5 * empty
+
+
+def test_messages_of_short_query_rings():
+    """The database messages of a query ring of 2^9, too short for words of four entries, cost less than 1.8 times
+    those of 2^10 in all of an encryption (2.2 times with words of four)."""
+    B.build()
+    W = synth.make_workload(n_eyes=1, n_db=2000, seed=21)
+    t = []
+    for log_n_q in (9, 10):
+        eng = E.Engine(log_n_db=12, log_n_q=log_n_q, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9).keygen()
+        t.append(_best_ms(lambda: eng.encrypt_db(W.db_codes, W.db_masks)))
+    assert t[0] < 1.8 * t[1]
