@@ -297,10 +297,32 @@ struct QEncArgs {
     const uint64_t *eye_ids;
     icm::NttMod nt[2];
     const ulonglong2 *shat;              // [nqblk][Lq][Nq]: transforms of s_{q,t}, times Nq^-1
+    uint32_t h;
+    const int32_t *sq_pos; const int8_t *sq_sgn;     // [nqblk][h]: the supports, for the direct form
     uint64_t q[ICM_MAX_LIMBS], dl[ICM_MAX_LIMBS];   // primes and Delta mod q_l
     uint32_t n_cols;
     uint64_t *ct;                        // [Lq][n_cols][K]
 };
+
+// Message coefficient k of rotation r of a masked code: x_s[row, col, b] = x[row, (col + s) mod 200, b] on
+// 16 x 200 x 4.
+__device__ __forceinline__ int rotated_bit(const QEncArgs &a, const uint8_t *code, const uint8_t *mask, uint32_t r, uint32_t k) {
+    if (k >= a.code_bits) return 0;
+    const int shift = (int)r - (int)(a.rho - 1) / 2;
+    const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
+    const uint32_t src = (row * 200 + (uint32_t)(((int)cc + shift + 200) % 200)) * 4 + b;
+    const int cb = template_bit(code, src), mb = template_bit(mask, src);
+    return mb - 2 * (cb & mb);
+}
+// b = -(s a) + Delta m + e of one coefficient, given sa = (s a) mod q
+__device__ __forceinline__ uint64_t query_b(const QEncArgs &a, uint32_t l, uint64_t sa, int m, uint64_t ke, uint64_t at) {
+    const uint64_t q = a.q[l];
+    uint64_t v = sa ? q - sa : 0;
+    if (m > 0) v = add_mod(v, a.dl[l], q);
+    else if (m < 0) v = sub_mod(v, a.dl[l], q);
+    const int err = cbd_sample(sm64(ke, at), a.eta);
+    return err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
+}
 
 // One block per (2^logc query columns, limb l < Lq): the same transforms as k_db_apart_b.  32 eyes
 // (992 columns, N_q = 2^13, two primes): 23.2 ms with h = 512 additions per coefficient, 1.24 ms with
@@ -348,32 +370,46 @@ __global__ void __launch_bounds__(NT_MUL, 1) k_query_encrypt(const __grid_consta
         for (uint32_t c = 0; c < C; ++c) {
             const uint32_t j = j0 + c, e = j / a.rho, r = j % a.rho;
             if (j >= a.n_cols) break;
-            const int shift = (int)r - (int)(a.rho - 1) / 2;
             const uint8_t *code = a.codes + (size_t)e * tb, *mask = a.masks + (size_t)e * tb;
             const uint64_t ke = stream_key(a.seed, ICM_KIND_E_Q, a.eye_ids[e], 0);
             uint64_t *ct = a.ct + ((size_t)l * a.n_cols + j) * a.K + (size_t)t * N;
             for (uint32_t i = threadIdx.x; i < N; i += NT_MUL) {
                 const uint32_t k = t * N + i;
                 const uint64_t sa = icm::sub_if(icm::sub_if(su[c * stride + icm::ntt_pad(i)], 2 * q), q);
-                uint64_t v = sa ? q - sa : 0;                      // -(s * a)
-                // rotated masked bit-vector: x_s[row, col, b] = x[row, (col + s) mod 200, b] on 16 x 200 x 4
-                int m = 0;
-                if (k < a.code_bits) {
-                    const uint32_t row = k / 800, cc = (k / 4) % 200, b = k % 4;
-                    const uint32_t src = (row * 200 + (uint32_t)(((int)cc + shift + 200) % 200)) * 4 + b;
-                    const int cb = template_bit(code, src), mb = template_bit(mask, src);
-                    m = mb - 2 * (cb & mb);
-                }
-                if (m > 0) v = add_mod(v, a.dl[l], q);
-                else if (m < 0) v = sub_mod(v, a.dl[l], q);
-                const int err = cbd_sample(sm64(ke, (uint64_t)r * a.d2 + k), a.eta);
-                v = err >= 0 ? add_mod(v, (uint64_t)err, q) : sub_mod(v, (uint64_t)(-err), q);
-                ct[i] = v;
+                ct[i] = query_b(a, l, sa, rotated_bit(a, code, mask, r, k), ke, (uint64_t)r * a.d2 + k);
             }
         }
         // Word c N + i is written by thread (c N + i) mod NT_MUL above and read by thread i mod NT_MUL here:
         // the same one unless a column is shorter than the block.
         if (N < NT_MUL) __syncthreads();
+    }
+}
+
+// The direct form, one block per (query column j, limb l < Lq): h additions per coefficient (query_direct).
+__global__ void __launch_bounds__(1024) k_query_encrypt_direct(const __grid_constant__ QEncArgs a) {
+    extern __shared__ uint64_t su[];                               // the column's a [Nq]
+    const uint32_t j = blockIdx.x, l = blockIdx.y, e = j / a.rho, r = j % a.rho, N = a.Nq, tb = a.code_bits / 8;
+    const uint64_t q = a.q[l];
+    const uint64_t ka = stream_key(a.seed, ICM_KIND_A_Q, a.eye_ids[e], l), ke = stream_key(a.seed, ICM_KIND_E_Q, a.eye_ids[e], 0);
+    const uint8_t *code = a.codes + (size_t)e * tb, *mask = a.masks + (size_t)e * tb;
+    uint64_t *ct = a.ct + ((size_t)l * a.n_cols + j) * a.K;
+    for (uint32_t i = threadIdx.x; i < N; i += blockDim.x) {
+        const uint64_t v = uniform_mod(sm64(ka, (uint64_t)r * N + i), q);
+        su[i] = v;
+        ct[a.d2 + i] = v;
+    }
+    __syncthreads();
+    for (uint32_t k = threadIdx.x; k < a.d2; k += blockDim.x) {
+        const uint32_t t = k / N, i = k % N;
+        uint64_t sa = 0;
+        for (uint32_t c = 0; c < a.h; ++c) {
+            const uint32_t p = (uint32_t)a.sq_pos[t * a.h + c];
+            const int s = a.sq_sgn[t * a.h + c];
+            const uint64_t term = (i >= p) ? su[i - p] : su[N + i - p];
+            const bool neg = (i >= p) ? (s < 0) : (s > 0);
+            sa = neg ? sub_mod(sa, term, q) : add_mod(sa, term, q);
+        }
+        ct[k] = query_b(a, l, sa, rotated_bit(a, code, mask, r, k), ke, (uint64_t)r * a.d2 + k);
     }
 }
 
@@ -431,7 +467,7 @@ namespace icm {
 
 cudaError_t encrypt_set_attributes() {
     return allow_smem(k_db_messages<false>, k_db_messages<true>, k_db_apart_b_direct, k_db_apart_b<8>, k_db_apart_b<16>, k_db_apart_b<32>,
-                      k_query_encrypt<8>, k_query_encrypt<16>, k_query_encrypt<32>, k_ntt_secret);
+                      k_query_encrypt_direct, k_query_encrypt<8>, k_query_encrypt<16>, k_query_encrypt<32>, k_ntt_secret);
 }
 
 cudaError_t launch_db_messages(const icm_ctx *c, const LayoutDev &lay, const uint8_t *d_codes,
@@ -507,6 +543,14 @@ cudaError_t launch_db_apart_and_b(const icm_ctx *c, const LayoutDev &lay, uint64
                     : wpt > 8 ? launch_mul(k_db_apart_b<16>, a, grid, smem, st) : launch_mul(k_db_apart_b<8>, a, grid, smem, st);
 }
 
+// Whether h additions per coefficient cost less than the transforms of a column (one forward, one inverse per
+// secret), per limb.  12 eyes, two primes, d2 = 2^14, us, additions / transforms: h = 16 N_q = 2^5 478 / 4,800, 2^7
+// 472 / 1,700, 2^9 472 / 695, 2^10 471 / 528, 2^13 482 / 568; h = 64 2^7 1,246 / 1,674, 2^8 1,248 / 1,008, 2^10
+// 1,242 / 528; h = 512 8,420 / 470 to 690.
+static bool query_direct(uint32_t h, uint32_t d2, uint32_t N) {
+    return (uint64_t)h * d2 < (uint64_t)(d2 / N + 1) * std::max(16 * N, 11500u);
+}
+
 cudaError_t launch_query_encrypt(const icm_ctx *c, const uint8_t *d_codes, const uint8_t *d_masks,
                                  const uint64_t *d_eye_ids, uint32_t n_eyes, uint64_t *d_ct, cudaStream_t st) {
     QEncArgs a{};
@@ -519,6 +563,11 @@ cudaError_t launch_query_encrypt(const icm_ctx *c, const uint8_t *d_codes, const
     a.ct = d_ct;
     if (a.n_cols == 0) return cudaSuccess;
     if (!a.shat) return cudaErrorInvalidValue;                           // rings above 2^14
+    if (query_direct(c->p.hamming_weight, a.d2, a.Nq)) {
+        a.h = c->p.hamming_weight; a.sq_pos = c->d_sq_pos; a.sq_sgn = c->d_sq_sgn;
+        k_query_encrypt_direct<<<dim3(a.n_cols, a.Lq), 1024, (size_t)a.Nq * 8, st>>>(a);
+        return cudaGetLastError();
+    }
     // two columns share their twiddles where there are enough of them to fill the SMs
     a.logc = mul_logc(a.Nq, a.n_cols * a.Lq >= 2 * 152 ? 2 : 1);
     const size_t smem = mul_smem(a.Nq, a.logc);

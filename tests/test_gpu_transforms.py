@@ -81,17 +81,18 @@ def test_decryption_large_rings(log_n_db, n_db):
     assert torch.equal(eng.decrypt(s).cpu(), want.round().long().cpu())
 
 
-# two columns of one block shorter than the block's 512 threads (n_eyes * 31 * Lq >= 304), one and two query primes,
-# an odd column count among them
-@pytest.mark.parametrize("log_n_q,L,Lq,n_eyes", [(5, 2, 1, 12), (5, 4, 2, 6), (7, 2, 1, 11), (7, 4, 2, 12), (8, 2, 1, 12),
-                                                 (8, 4, 2, 5), (9, 4, 2, 12)])
-def test_query_encryption_two_short_columns(log_n_q, L, Lq, n_eyes):
+# rings of which two columns in one block are shorter than its 512 threads (n_eyes * 31 * Lq >= 304), one and two query
+# primes, an odd column count among them: by additions (h = 16) and by transforms
+@pytest.mark.parametrize("log_n_q,h,L,Lq,n_eyes", [(5, 16, 2, 1, 12), (5, 16, 4, 2, 6), (7, 16, 2, 1, 11), (7, 128, 2, 1, 11),
+                                                   (7, 128, 4, 2, 12), (8, 16, 4, 2, 5), (8, 64, 2, 1, 12), (8, 128, 4, 2, 5),
+                                                   (9, 16, 4, 2, 12), (9, 64, 4, 2, 12), (10, 16, 2, 1, 12), (13, 16, 2, 1, 1)])
+def test_query_encryption_short_columns(log_n_q, h, L, Lq, n_eyes):
     B.build()
-    prm = dict(log_n_db=5, log_n_q=log_n_q, n_limbs=L, n_limbs_q=Lq, prime_bits=60, log2_delta=60 if Lq == 2 else 40,
+    prm = dict(log_n_db=7, log_n_q=log_n_q, n_limbs=L, n_limbs_q=Lq, prime_bits=60, log2_delta=60 if Lq == 2 else 40,
                seed=9)
-    P = O.Params(**prm, h=16)
+    P = O.Params(**prm, h=h)
     W = synth.make_workload(n_eyes=n_eyes, n_db=1, seed=21)
-    eng = E.Engine(**prm, hamming_weight=16).keygen()
+    eng = E.Engine(**prm, hamming_weight=h).keygen()
     ct = O.query_encrypt(P, W.q_codes, W.q_masks, W.eye_ids)
     for _ in range(3):
         assert np.array_equal(_u64(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), ct.shape), ct)
@@ -206,3 +207,16 @@ def test_messages_of_short_query_rings():
         eng = E.Engine(log_n_db=12, log_n_q=log_n_q, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9).keygen()
         t.append(_best_ms(lambda: eng.encrypt_db(W.db_codes, W.db_masks)))
     assert t[0] < 1.8 * t[1]
+
+
+def test_short_query_rings_cost_what_long_ones_do():
+    """With few non-zeros in the secrets the additions of a query encryption do not depend on the ring; transforms
+    over rings of 2^6 would take six times those over 2^13."""
+    B.build()
+    W = synth.make_workload(n_eyes=12, n_db=1, seed=21)
+    t = []
+    for log_n_q in (6, 13):
+        eng = E.Engine(log_n_db=6, log_n_q=log_n_q, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40, seed=9,
+                       hamming_weight=16).keygen()
+        t.append(_best_ms(lambda: eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids)))
+    assert t[0] < 2.5 * t[1]
