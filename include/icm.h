@@ -119,7 +119,7 @@ icm_status icm_ctx_crt_moduli(const icm_ctx *ctx, int32_t *moduli, size_t cap, s
 /* Key generation (Section 2.2.2 refers to the CKKS paper): samples the database secrets
  * s_{db,t} (degree N_db) and query secrets s_{q,t} (degree N_q) as sparse ternary polynomials
  * with exactly h non-zeros from the context seed, and uploads their supports to the current
- * device.  Secrets never leave the library. */
+ * device.  Secrets never leave the library.  A further call on the same device changes nothing. */
 icm_status icm_keygen(icm_ctx *ctx);
 
 /* ---------------------------------------------------------------- database (setup) ---- */

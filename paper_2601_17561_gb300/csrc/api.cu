@@ -275,6 +275,10 @@ icm_status icm_keygen(icm_ctx *c) {
     if (!c) return fail(ICM_EINVAL, "null context");
     int dev = 0;
     CUDA_TRY(cudaGetDevice(&dev));
+    // Supports and transforms depend on the parameters alone (the secrets are drawn from the seed): a further call
+    // on the same device has nothing to do and leaves them where captured graphs read them.  A call that
+    // fails leaves the keys as they were.
+    if (c->have_keys && c->device == dev) return ICM_OK;
     const uint32_t h = c->p.hamming_weight;
     // database secrets for up to 2^17 / N_db blocks plus one (a chunk of up to 2^17 + N_db templates)
     const uint32_t max_blocks = (1u << 17) / c->N_db + 2;
@@ -304,35 +308,29 @@ icm_status icm_keygen(icm_ctx *c) {
         return fail(ICM_ECUDA, std::string("keygen upload: ") + cudaGetErrorString(e));
     }
     // shared-memory opt-ins are set here, outside any stream capture
-    e = encrypt_set_attributes();
+    e = crt_set_attributes();
+    if (e == cudaSuccess) e = encrypt_set_attributes();
     if (e == cudaSuccess) e = decrypt_set_attributes();
     if (e == cudaSuccess) e = slots_set_attributes();
     if (e != cudaSuccess) {
         cudaFree(a); cudaFree(b); cudaFree(x); cudaFree(y);
         return fail(ICM_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
     }
-    // The transforms depend on the parameters alone (the secrets are drawn from the seed): a further call on
-    // the same device keeps them where captured graphs read them, and a call that fails leaves the keys as
-    // they were.
-    if (!c->have_keys || c->device != dev) {
-        NttSet nt;
-        std::string why;
-        e = build_ntt(c, a, x, max_blocks, b, y, nt, why);
-        if (e != cudaSuccess) {
-            nt.release();
-            cudaFree(a); cudaFree(b); cudaFree(x); cudaFree(y);
-            return fail(ICM_ECUDA, "keygen transforms: " + (why.empty() ? cudaGetErrorString(e) : why));
-        }
-        c->nt.release();
-        c->nt = nt;
+    NttSet nt;
+    std::string why;
+    e = build_ntt(c, a, x, max_blocks, b, y, nt, why);
+    if (e != cudaSuccess) {
+        nt.release();
+        cudaFree(a); cudaFree(b); cudaFree(x); cudaFree(y);
+        return fail(ICM_ECUDA, "keygen transforms: " + (why.empty() ? cudaGetErrorString(e) : why));
     }
+    c->nt.release();
+    c->nt = nt;
     if (c->d_sdb_pos) { cudaFree(c->d_sdb_pos); cudaFree(c->d_sdb_sgn); cudaFree(c->d_sq_pos); cudaFree(c->d_sq_sgn); }
     c->d_sdb_pos = a; c->d_sdb_sgn = x; c->d_sq_pos = b; c->d_sq_sgn = y;
     c->max_db_blocks = max_blocks;
     c->device = dev;
     c->have_keys = true;
-    e = crt_set_attributes();
-    if (e != cudaSuccess) return fail(ICM_ECUDA, std::string("kernel attributes: ") + cudaGetErrorString(e));
     return ICM_OK;
 }
 
