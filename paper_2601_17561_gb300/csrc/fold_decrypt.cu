@@ -95,7 +95,58 @@ struct DecArgs {
     const uint64_t *sc;    // [L][n_cols][M]
     int64_t *num;          // [n_cols][n_real]
     uint32_t *err_bits;    // optional: max |x - round(x)| over all outputs, as fp32 bits
+    uint32_t h;
+    const int32_t *sdb_pos; const int8_t *sdb_sgn;   // [blocks][h]: the supports, for the direct form
 };
+
+// F = sum_l y_l floor(2^128 / q_l) mod 2^128: adds y (rhi 2^64 + rlo)
+__device__ __forceinline__ void crt_add(const icm::CrtDecode &crt, uint32_t l, uint64_t y, uint64_t &fhi, uint64_t &flo) {
+    const uint64_t plo = y * crt.rlo[l];
+    const uint64_t phi = __umul64hi(y, crt.rlo[l]) + y * crt.rhi[l];
+    const uint64_t nlo = flo + plo;
+    fhi = fhi + phi + (nlo < flo ? 1 : 0);
+    flo = nlo;
+}
+// Numerator r of column j from F: F / 2^128 is D / Q_db modulo 1; as a signed 128-bit number it is the
+// centred value.
+__device__ __forceinline__ void decode(const DecArgs &a, uint32_t j, uint64_t r, uint64_t fhi, uint64_t flo) {
+    const double frac = (double)(int64_t)fhi * 0x1p-64 + (double)flo * 0x1p-128;
+    const double x = frac * a.crt.q_over_delta;
+    const double n = rint(x);
+    a.num[(size_t)j * a.lay.n_real + r] = (int64_t)n;
+    if (a.err_bits) {
+        // distance of the decoded value from the integer it rounds to (numerator units); the
+        // bits of non-negative floats order like unsigned integers
+        const uint32_t act = __activemask();
+        const uint32_t e = __reduce_max_sync(act, __float_as_uint((float)fabs(x - n)));
+        if ((threadIdx.x & 31) == (__ffs(act) - 1)) atomicMax(a.err_bits, e);
+    }
+}
+
+// The direct form, grid (ceil(n_real / 256), n_cols): one thread per (column, real database row), h additions
+// per limb from L2.  decrypt_direct says where that is the cheaper one.
+__global__ void __launch_bounds__(256) k_decrypt_direct(const __grid_constant__ DecArgs a) {
+    const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t j = blockIdx.y, N = a.lay.N;
+    if (r >= a.lay.n_real) return;
+    const uint32_t t = (uint32_t)(r / N), i = (uint32_t)(r % N);
+    const int64_t pos = pos_of(a.lay, (int)t, i);
+    uint64_t fhi = 0, flo = 0;
+    for (uint32_t l = 0; l < a.L; ++l) {
+        const uint64_t q = a.nt[l].q;
+        const uint64_t *col = a.sc + ((size_t)l * a.n_cols + j) * a.lay.M;
+        uint64_t d = col[pos];
+        for (uint32_t c = 0; c < a.h; ++c) {
+            const uint32_t p = (uint32_t)a.sdb_pos[t * a.h + c];
+            const int s = a.sdb_sgn[t * a.h + c];
+            const uint64_t term = (i >= p) ? col[i - p] : col[N + i - p];
+            const bool neg = (i >= p) ? (s < 0) : (s > 0);
+            d = neg ? sub_mod(d, term, q) : add_mod(d, term, q);
+        }
+        crt_add(a.crt, l, mulmod_shoup(d, a.crt.inv[l], a.crt.invs[l], q), fhi, flo);
+    }
+    decode(a, j, r, fhi, flo);
+}
 
 __device__ __forceinline__ void cluster_barrier() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -159,28 +210,9 @@ __global__ void __launch_bounds__(NT, MB) k_decrypt(const __grid_constant__ DecA
         __syncwarp();
         cluster_barrier();
         for (uint32_t i = l * NT + threadIdx.x; i < rows; i += a.L * NT) {
-            uint64_t fhi = 0, flo = 0;                  // sum_l y_l floor(2^128 / q_l) mod 2^128
-            for (uint32_t k = 0; k < a.L; ++k) {
-                const uint64_t y = ld_cluster(su_addr + icm::ntt_pad(i) * 8, k);
-                // y * (rhi 2^64 + rlo) mod 2^128
-                const uint64_t plo = y * a.crt.rlo[k];
-                const uint64_t phi = __umul64hi(y, a.crt.rlo[k]) + y * a.crt.rhi[k];
-                const uint64_t nlo = flo + plo;
-                fhi = fhi + phi + (nlo < flo ? 1 : 0);
-                flo = nlo;
-            }
-            // F / 2^128 is D / Q_db modulo 1; as a signed 128-bit number it is the centred value.
-            const double frac = (double)(int64_t)fhi * 0x1p-64 + (double)flo * 0x1p-128;
-            const double x = frac * a.crt.q_over_delta;
-            const double n = rint(x);
-            a.num[(size_t)j * a.lay.n_real + r0 + i] = (int64_t)n;
-            if (a.err_bits) {
-                // distance of the decoded value from the integer it rounds to (numerator units); the
-                // bits of non-negative floats order like unsigned integers
-                const uint32_t act = __activemask();
-                const uint32_t e = __reduce_max_sync(act, __float_as_uint((float)fabs(x - n)));
-                if ((threadIdx.x & 31) == (__ffs(act) - 1)) atomicMax(a.err_bits, e);
-            }
+            uint64_t fhi = 0, flo = 0;
+            for (uint32_t k = 0; k < a.L; ++k) crt_add(a.crt, k, ld_cluster(su_addr + icm::ntt_pad(i) * 8, k), fhi, flo);
+            decode(a, j, r0 + i, fhi, flo);
         }
         __syncwarp();
         cluster_barrier();                              // the limbs are read before the next block's product
@@ -277,6 +309,20 @@ cudaError_t decrypt_set_attributes() {
                       k_decrypt<32, 256, 2>, k_decrypt<16, 1024, 1>);
 }
 
+// Whether h additions per row and limb take less time than the transforms.  Both sides in us, fitted to
+// measurements at L = 4 (2 to 248 columns, 10 to 3,000 rows, N = 2^5 to 2^14, h = 16 to 512): the additions run
+// at 1.4 ps each, but no faster than a row's chain of them; the transforms by columns and limbs, but no faster
+// than a block of a cluster.  248 columns, us, additions / transforms: N = 2^14, h = 64, 1,000 rows 142 / 443;
+// 2^13, 100 rows 69 / 202; 2^12 65 / 100, 3,000 rows 299 / 116; 2^7, 3,000 rows, h = 16 93 / 396; h = 512, 3,000
+// rows 2^12 2,157 / 115, 100 rows 2^14 660 / 423.
+static bool decrypt_direct(uint32_t h, uint32_t N, uint32_t L, uint64_t rows, uint32_t n_cols) {
+    const double n = N, w = (double)n_cols * L, blocks = (double)((rows + N - 1) / N);
+    const double direct = (double)h * L * std::max(1.4e-6 * (double)rows * n_cols, 0.1 + 5e-6 * n);
+    const double transforms = blocks <= 1 ? n * std::max(2.2e-5 * w, 2.9e-3)
+                                          : (blocks + 1) * std::max(w * (0.0135 + 7e-6 * n), 3.6 + 7e-4 * n);
+    return direct < transforms;
+}
+
 cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_t *d_scores, uint32_t n_cols,
                            bool rescaled, int64_t *d_num, cudaStream_t st, uint32_t *d_err_bits) {
     DecArgs a{};
@@ -288,6 +334,11 @@ cudaError_t launch_decrypt(const icm_ctx *c, const LayoutDev &lay, const uint64_
     a.sc = d_scores; a.num = d_num; a.err_bits = d_err_bits;
     if (n_cols == 0 || lay.n_real == 0) return cudaSuccess;
     if (!a.shat) return cudaErrorInvalidValue;                           // rings above 2^14
+    if (decrypt_direct(c->p.hamming_weight, lay.N, a.L, lay.n_real, n_cols)) {
+        a.h = c->p.hamming_weight; a.sdb_pos = c->d_sdb_pos; a.sdb_sgn = c->d_sdb_sgn;
+        k_decrypt_direct<<<dim3((unsigned)((lay.n_real + 255) / 256), n_cols), 256, 0, st>>>(a);
+        return cudaGetLastError();
+    }
     const size_t smem = (size_t)ntt_words(lay.N) * 8;
     auto run = [&](auto kern, int nt) {
         cudaLaunchConfig_t cfg = {};

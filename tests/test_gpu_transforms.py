@@ -220,3 +220,42 @@ def test_short_query_rings_cost_what_long_ones_do():
                        hamming_weight=16).keygen()
         t.append(_best_ms(lambda: eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids)))
     assert t[0] < 2.5 * t[1]
+
+
+@pytest.mark.parametrize("log_n_db,h,n_db,n_eyes", [(7, 128, 300, 1), (8, 256, 700, 2), (9, 512, 40, 1), (10, 512, 2100, 3),
+                                                    (12, 512, 4100, 1), (12, 16, 4100, 2), (13, 64, 100, 2)])
+def test_decryption_routes(log_n_db, h, n_db, n_eyes):
+    """Small rings by transforms (many non-zeros in the secrets) and large ones by additions (few), one and several
+    blocks: the cleartext inner products at both levels, with the same error bound."""
+    B.build()
+    eng = E.Engine(log_n_db=log_n_db, log_n_q=9 if h > 256 else 8, n_limbs=2, n_limbs_q=1, prime_bits=60, log2_delta=40,
+                   seed=9, hamming_weight=h).keygen()
+    W = synth.make_workload(n_eyes=n_eyes, n_db=n_db, seed=21)
+    db = eng.encrypt_db(W.db_codes, W.db_masks)
+    s = eng.match(db, eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), n_eyes, "f16_crt"))
+
+    def signed(codes, masks):      # +1 / -1 where the mask is set, else 0: sums below 2^24 are exact in fp32
+        c, m = (torch.as_tensor(np.asarray(x)).cuda().float() for x in (codes, masks))
+        return m - 2 * c * m
+
+    rc, rm = O.rotated_templates(W.q_codes, W.q_masks, eng.rho)
+    want = (signed(rc, rm) @ signed(O.unpack(W.db_codes), O.unpack(W.db_masks)).T).round().long()
+    for scores in (s, eng.rescale(s)):
+        got, err = eng.decrypt(scores, with_error=True)
+        assert torch.equal(got, want) and 0 <= float(err) < 0.25
+
+
+def test_decryption_of_few_rows_in_a_large_ring():
+    """With few non-zeros in the secrets a decryption costs its rows, not its ring (4.2 times as much from N_db = 2^12
+    to 2^14 by transforms)."""
+    B.build()
+    W = synth.make_workload(n_eyes=8, n_db=100, seed=21)
+    t = []
+    for log_n_db in (12, 14):
+        eng = E.Engine(log_n_db=log_n_db, log_n_q=9, n_limbs=4, n_limbs_q=2, prime_bits=60, log2_delta=60, seed=9,
+                       hamming_weight=64).keygen()
+        s = eng.match(eng.encrypt_db(W.db_codes, W.db_masks),
+                      eng.prepare(eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids), 8, "f16_crt"))
+        t.append(_best_ms(lambda: eng.decrypt(s)))
+        s = None
+    assert t[1] < 2.5 * t[0]
