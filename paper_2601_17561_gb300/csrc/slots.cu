@@ -455,8 +455,8 @@ int sm_count() {
 }  // namespace
 
 cudaError_t slots_set_attributes() {
-    return allow_smem(k_slot_db_encode, k_mu_encode, k_ntt_fwd<512>, k_ntt_fwd<1024>, k_ntt_mul_inv<512>,
-                      k_ntt_mul_inv<1024>, k_slot_dec_limbs, k_slot_decode);
+    return allow_smem(k_slot_db_encode, k_mu_encode, k_ntt_fwd<128>, k_ntt_fwd<512>, k_ntt_fwd<1024>, k_ntt_mul_inv<128>,
+                      k_ntt_mul_inv<512>, k_ntt_mul_inv<1024>, k_slot_dec_limbs, k_slot_decode);
 }
 
 // Workspace layout of icm_normalize (offsets 256-byte aligned): rotated query masks [n_cols][1600],
@@ -639,12 +639,14 @@ icm_status icm_normalize(icm_ctx *c, const icm_scores *in, const uint8_t *dev_q_
     // 3. NTT of every mu (in place) and of every a-part
     if (!c->nt.tab_db) return sfail(ICM_EINVAL, "icm_keygen has not run");
     const size_t psm = (size_t)ntt_words(N) * 8;
-    // one polynomial per block in shared memory, as many blocks per SM as fit
-    const unsigned per_sm = (unsigned)std::max<size_t>(1, std::min<size_t>(4, (size_t)220 * 1024 / psm));
-    // 64 registers allow 1,024 threads per SM: two blocks, or one larger where only one polynomial fits
-    const unsigned ntt_threads = per_sm > 1 ? 512 : 1024;
-    auto *const fwd = per_sm > 1 ? k_ntt_fwd<512> : k_ntt_fwd<1024>;
-    auto *const mul_inv = per_sm > 1 ? k_ntt_mul_inv<512> : k_ntt_mul_inv<1024>;
+    // one polynomial per block in shared memory; 64 registers allow 1,024 threads per SM: one block where only one
+    // polynomial fits, two of 512 threads, or eight of 128 in rings with fewer than 128 groups of eight elements
+    // (500 templates, 32 eyes: N_db = 2^7 448 us, 820 with 512 threads; 2^8 328 and 524, 2^9 306 and 428)
+    const unsigned fit = (unsigned)((size_t)220 * 1024 / psm);
+    const unsigned ntt_threads = N <= 512 ? 128 : fit > 1 ? 512 : 1024;
+    const unsigned per_sm = N <= 512 ? 8 : std::max(1u, std::min(4u, fit));
+    auto *const fwd = N <= 512 ? k_ntt_fwd<128> : fit > 1 ? k_ntt_fwd<512> : k_ntt_fwd<1024>;
+    auto *const mul_inv = N <= 512 ? k_ntt_mul_inv<128> : fit > 1 ? k_ntt_mul_inv<512> : k_ntt_mul_inv<1024>;
     {
         FwdArgs a{};
         for (uint32_t l = 0; l < Lq; ++l) a.nt[l] = c->nt.db[l];

@@ -259,3 +259,36 @@ def test_decryption_of_few_rows_in_a_large_ring():
         t.append(_best_ms(lambda: eng.decrypt(s)))
         s = None
     assert t[1] < 2.5 * t[0]
+
+
+def _normalised(log_n_db, n_db, n_eyes):
+    eng = E.Engine(log_n_db=log_n_db, log_n_q=9, n_limbs=4, n_limbs_q=2, prime_bits=60, log2_delta=60, seed=9,
+                   hamming_weight=16).keygen()
+    W = synth.make_workload(n_eyes=n_eyes, n_db=n_db, seed=21)
+    db = eng.encrypt_db_slots(W.db_codes, W.db_masks)
+    ct = eng.encrypt_query(W.q_codes, W.q_masks, W.eye_ids)
+    r = eng.rescale(eng.match(db, eng.prepare(ct, n_eyes, "f16_crt")))
+    return eng, W, r, torch.as_tensor(W.q_masks).cuda(), torch.as_tensor(W.db_masks).cuda()
+
+
+@pytest.mark.parametrize("log_n_db", [5, 7, 9, 10])
+def test_normalisation_of_small_rings(log_n_db):
+    """Blocks of 128 threads (rings up to 2^9) and of 512: decoded distances of all the blocks, a partial last
+    one among them."""
+    B.build()
+    eng, W, r, qm, dm = _normalised(log_n_db, 777, 2)
+    hd = eng.decrypt_slots(r, eng.normalize(r, qm, dm)).cpu().numpy()
+    rc, rm = O.rotated_templates(W.q_codes, W.q_masks, eng.rho)
+    ref = O.fractional_hd(*O.hd_counts(rc, rm, O.unpack(W.db_codes), O.unpack(W.db_masks)))
+    assert hd.shape == ref.shape and np.abs(hd - ref).max() < 1e-4
+
+
+def test_normalisation_time_of_small_rings():
+    """The same scores in rings of 2^7 and 2^9 take about the same time (1.9 times with blocks of 512 threads)."""
+    B.build()
+    t = []
+    for log_n_db in (7, 9):
+        eng, _, r, qm, dm = _normalised(log_n_db, 500, 32)
+        out = eng.normalize(r, qm, dm)
+        t.append(_best_ms(lambda: eng.normalize(r, qm, dm, out=out)))
+    assert t[0] < 1.7 * t[1]
