@@ -178,13 +178,23 @@ __global__ void __launch_bounds__(NT, 1) k_crt_p1(P1Args p) {
         }
     };
     constexpr int CH = ROWB / 16;                 // 16-byte chunks per column per slab
+    // fp16 planes: offsets of this thread's columns (crt_f16_off at its k of slab 0), in chunks; a slab of KS is
+    // KS / 16 blocks of G tiles further (G: column groups of the round).  (Worked out for every chunk, 31 columns
+    // x 8,322 rows, 4 limbs, K = 24,576 took 54.6 ms for 49.5, 992 columns 232.8 for 205.6.)
+    static_assert(NT % CH == 0 && KS % 16 == 0, "a thread keeps its chunk of k");
+    constexpr int NB = BN * CH / NT;
+    uint32_t b_off[F16 ? NB : 1];
+    const uint32_t b_slab = KS / 16 * (2048 / 8) * icm::crt_f16_groups(p.n0 + nb, N);
+    if (F16)
+#pragma unroll
+        for (int e = 0; e < NB; ++e)
+            b_off[e] = (uint32_t)(icm::crt_f16_off(p.n0 + nb + (tid + e * NT) / CH, (uint64_t)(tid % CH) * 8, N, Kp) / 8);
     auto load_b = [&](int st, uint64_t k0) {
 #pragma unroll
-        for (int e = 0; e < (BN * CH) / NT; ++e) {
+        for (int e = 0; e < NB; ++e) {
             const int idx = tid + e * NT, col = idx / CH, ch = idx % CH;
             const bool ok = p.n0 + nb + col < N && nb + col < p.nch;
-            const uint64_t off = F16 ? icm::crt_f16_off(p.n0 + nb + col, k0 + ch * 8, N, Kp) * 2
-                                     : ((nb + col) * Kp + k0) * ESZ + ch * 16;
+            const uint64_t off = F16 ? (uint64_t)(b_off[e] + (uint32_t)(k0 / KS) * b_slab) * 16 : ((nb + col) * Kp + k0) * ESZ + ch * 16;
             const unsigned char *src = Bl + (ok ? off : 0);
             cp_async16(smem_u32(sB + (size_t)st * BN * LDB + col * LDB + ch * 16), src, ok);
         }

@@ -95,13 +95,16 @@ __host__ __device__ inline uint64_t crt_f16_ncols(uint64_t N) { return (N + CRT_
 inline uint64_t crt_plane_bytes(bool f16, uint32_t n_limbs, uint32_t n_mod, uint64_t N, uint64_t Kp) {
     return f16 ? (uint64_t)n_limbs * n_mod * crt_f16_ncols(N) * Kp * 2 : (uint64_t)n_limbs * n_mod * N * Kp;
 }
+// column groups of 256 of column j's round
+__host__ __device__ __forceinline__ uint32_t crt_f16_groups(uint64_t j, uint64_t N) {
+    const uint64_t left = crt_f16_ncols(N) - (j & ~1023ull);
+    return left < 1024 ? (uint32_t)(left >> 8) : 4u;
+}
 // fp16 element offset of (column j, k) within one (limb, modulus) plane of N columns and Kp of K
 // (Kp a multiple of 16)
 __host__ __device__ __forceinline__ uint64_t crt_f16_off(uint64_t j, uint64_t k, uint64_t N, uint64_t Kp) {
     const uint64_t r0 = j & ~1023ull;                                    // first column of the round
-    const uint64_t left = crt_f16_ncols(N) - r0;
-    const uint32_t G = left < 1024 ? (uint32_t)(left >> 8) : 4u;
-    const uint32_t jj = (uint32_t)(j & 1023), half = jj >= 128 * G ? 1u : 0u, c = jj - half * 128 * G;
+    const uint32_t G = crt_f16_groups(j, N), jj = (uint32_t)(j & 1023), half = jj >= 128 * G ? 1u : 0u, c = jj - half * 128 * G;
     return r0 * Kp + ((half * (Kp >> 4) + (k >> 4)) * G + (c >> 7)) * 2048 + ((k >> 3) & 1) * 1024 +
            ((c & 127) >> 3) * 64 + (c & 7) * 8 + (k & 7);
 }
