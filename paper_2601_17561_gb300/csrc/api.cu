@@ -837,11 +837,18 @@ icm_status icm_ppmm(icm_form form, const uint64_t *q, uint32_t n_limbs, const ui
             const size_t pl = crt_plane_bytes(f16, n_limbs, k.n_mod, N, i8_kpad(K));
             const size_t sc = crt_scratch_bytes(n_limbs, k.n_mod, N, M);
             if ((pl || sc) && (!dev_ws || ws_bytes < align256(pl) + sc)) return fail(ICM_ENOMEM, "workspace too small");
+            // fp16: the tcgen05 kernel (3 x 3001 x 500 x 8192: 1.50 ms, 12.0 on mma.sync) where K and the
+            // operand's alignment allow it, but not for short products of one wave, whose time is the
+            // launches' (L x M x N x K, us, mma.sync / tcgen05: 1 x 300 x 300 x 64 61 / 76, x 192 72 / 76, x 256 79 / 78;
+            // 1 x 1 x 1 x 2 45 / 49, x 128 52 / 52; two waves, 1 x 1000 x 300 x 2 79 / 78)
+            int dev = 0, sms = 0;
+            cudaGetDevice(&dev);
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            const uint64_t tiles = (uint64_t)n_limbs * k.n_mod * ((M + 127) / 128) * ((N + 255) / 256);
+            const bool tc = f16 && (K > 192 || tiles > (uint64_t)sms);
             e = launch_crt_planes(f16, k, dev_B, N, dev_ws, N, K, i8_kpad(K), (cudaStream_t)stream);
             if (e == cudaSuccess)
-                // fp16: the tcgen05 kernel (3 x 3001 x 500 x 8192: 2.05 ms, 12.0 ms on mma.sync) where K and
-                // the operand's alignment allow it
-                e = launch_ppmm_crt(f16, f16 ? 2 : 256, k, dev_A, false, dev_ws, dev_C, M, N, K, i8_kpad(K),
+                e = launch_ppmm_crt(f16, tc ? 2 : 256, k, dev_A, false, dev_ws, dev_C, M, N, K, i8_kpad(K),
                                     (char *)dev_ws + align256(pl), (cudaStream_t)stream);
             break;
         }

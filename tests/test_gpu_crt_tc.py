@@ -161,3 +161,40 @@ def test_digits_beside_residues(rows, n_eyes, launches):
     C.icm_device_status(True)
     for a, b in zip(*res):
         assert np.array_equal(a, b)
+
+
+def _ppmm_operands(M, N, K):
+    q = [(1 << 60) - 93, (1 << 50) - 27, (1 << 31) - 1]
+    g = torch.Generator(device="cuda").manual_seed(M + N + K)
+    A, Bm = (torch.stack([torch.randint(0, x, (n, K), generator=g, device="cuda", dtype=torch.int64) for x in q])
+             for n in (M, N))
+    return q, A, Bm
+
+
+@pytest.mark.parametrize("M,N,K", [(1, 1, 192), (1, 1, 194), (100, 31, 192), (100, 31, 194), (300, 300, 2), (2000, 300, 2)])
+def test_ppmm_short_products(M, N, K):
+    """Both sides of the line between mma.sync and tcgen05 for short products, equal to the u64 form."""
+    q, A, Bm = _ppmm_operands(M, N, K)
+    assert torch.equal(E.ppmm("f16_crt", q, A, Bm), E.ppmm("u64", q, A, Bm))
+
+
+def test_ppmm_short_product_time():
+    """A short product of one wave takes the time that it takes with an odd K, which mma.sync computes (1.2 times it
+    on tcgen05)."""
+    B.build()
+    t = {}
+    for K in (63, 64):
+        q, A, Bm = _ppmm_operands(300, 300, K)
+        q, A, Bm = q[:1], A[:1].contiguous(), Bm[:1].contiguous()
+        Cm = torch.empty((1, 300, 300), dtype=torch.int64, device="cuda")
+        wb = C.icm_ppmm_workspace_bytes(C.FORMS["f16_crt"], 1, 300, 300, K)
+        ws, ts = torch.empty(wb, dtype=torch.uint8, device="cuda"), []
+        for _ in range(100):
+            a, b = torch.cuda.Event(True), torch.cuda.Event(True)
+            a.record()
+            C.icm_ppmm(C.FORMS["f16_crt"], q, 1, A, Bm, Cm, 300, 300, K, ws, wb)
+            b.record()
+            torch.cuda.synchronize()
+            ts.append(a.elapsed_time(b))
+        t[K] = min(ts)
+    assert t[64] < 1.15 * t[63]
