@@ -803,7 +803,8 @@ icm_status icm_ppmm(icm_form form, const uint64_t *q, uint32_t n_limbs, const ui
         if (!make_i8_consts(form, qv.data(), qv.size(), K, kp2, &why)) return fail(ICM_EINVAL, why);
     }
     const LimbTable lt = make_limb_table(qv);
-    if (crt_set_attributes() != cudaSuccess) return fail(ICM_ECUDA, "kernel attributes");
+    if ((form == ICM_FORM_I8_CRT || form == ICM_FORM_F16_CRT) && crt_set_attributes() != cudaSuccess)
+        return fail(ICM_ECUDA, "kernel attributes");
     cudaError_t e;
     switch (form) {
         case ICM_FORM_U64: e = launch_ppmm_u64(lt, dev_A, dev_B, dev_C, M, N, K, false, (cudaStream_t)stream); break;
