@@ -320,7 +320,8 @@ icm_status icm_device_status(int clear);
 /* Autotuner: times the kernel variants of the CRT product that apply on the caller's batch (one
  * icm_match_batch per variant, CUDA events on `stream`): the tcgen05 variants 1-3 for the fp16
  * form with an even K, else the mma.sync tiles 128 and 256.  Keeps the fastest for the context
- * and reports it (0 for forms with a single variant).  ms_per_choice (optional, n_choices
+ * and reports it (0 for forms with a single variant); a query whose columns are all multiplied as
+ * digits runs one kernel under all the tcgen05 variants and leaves the context's choice as it is.  ms_per_choice (optional, n_choices
  * entries) receives the time of each variant in the fixed order 128, 256, 1, 2, 3, with 0 for the
  * variants not timed. */
 icm_status icm_autotune(icm_ctx *ctx, const icm_db *const *dbs, size_t n_dbs, const icm_query *q,

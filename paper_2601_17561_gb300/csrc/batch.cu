@@ -156,8 +156,11 @@ icm_status icm_autotune(icm_ctx *c, const icm_db *const *dbs, size_t n_dbs, cons
     // ms_per_choice keeps the fixed order 128, 256, 1, 2, 3 (0 for variants not timed)
     const int choices[5] = {128, 256, 1, 2, 3};
     const bool tc = q->form == ICM_FORM_F16_CRT && crt_tc_supported(c->K);
+    // a query whose columns are all digits runs the same kernel under every tcgen05 variant: the times say
+    // nothing about them, and the context's choice stands for wider queries
+    const bool choose = !tc || q->n_crt > 0;
     float best_ms = 1e30f;
-    int best = c->crt_bn;
+    int best = tc && !crt_tc_variant(c->crt_bn) ? ICM_CRT_TCGEN05_DEFAULT : c->crt_bn;
     cudaStream_t st = (cudaStream_t)stream;
     cudaEvent_t a, b;
     cudaEventCreate(&a);
@@ -178,7 +181,7 @@ icm_status icm_autotune(icm_ctx *c, const icm_db *const *dbs, size_t n_dbs, cons
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, a, b);
         if (e != cudaSuccess) { s = api_fail(ICM_ECUDA, cudaGetErrorString(e)); break; }
         if (ms_per_choice && (size_t)i < n_choices) ms_per_choice[i] = ms;
-        if (ms < best_ms) { best_ms = ms; best = choices[i]; }
+        if (choose && ms < best_ms) { best_ms = ms; best = choices[i]; }
     }
     cudaEventDestroy(a);
     cudaEventDestroy(b);

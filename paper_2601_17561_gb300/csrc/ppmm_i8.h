@@ -63,6 +63,7 @@ cudaError_t crt_set_attributes();
 // moduli in groups of six, 3 = with the wave bound and all moduli in one group.
 #define ICM_CRT_TCGEN05 1
 #define ICM_CRT_TCGEN05_LAST 3
+#define ICM_CRT_TCGEN05_DEFAULT 2
 inline bool crt_tc_variant(int v) { return v >= ICM_CRT_TCGEN05 && v <= ICM_CRT_TCGEN05_LAST; }
 cudaError_t launch_crt_combine(const I8Consts &k, const ChunkTab &tab, const void *scratch, uint64_t N, uint64_t n0,
                                uint64_t nch, cudaStream_t st);

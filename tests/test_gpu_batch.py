@@ -133,3 +133,18 @@ def test_graph_replay_tcgen05_variant(setup, variant):
         del plan
     finally:
         C.icm_ctx_set_variant(eng.ctx, 0)
+
+
+def test_autotune_on_digit_columns_keeps_the_variant(setup):
+    """One eye's columns are all multiplied as digits, by one kernel under every tcgen05 variant: the tuner has
+    nothing to choose by and leaves the context's variant for the batches that follow."""
+    from paper_2601_17561_gb300 import icm as C
+    W, eng, dbs = setup["W"], setup["eng"], setup["dbs"]
+    q = eng.prepare(eng.encrypt_query(W.q_codes[:1], W.q_masks[:1], W.eye_ids[:1]), 1, "f16_crt")
+    try:
+        for v in (1, 2, 3, 2, 1, 3):
+            C.icm_ctx_set_variant(eng.ctx, v)
+            best, ms = eng.autotune(dbs, q)
+            assert best == v and all(m > 0 for m in ms[2:5])
+    finally:
+        C.icm_ctx_set_variant(eng.ctx, 0)
