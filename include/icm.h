@@ -186,10 +186,10 @@ icm_status icm_scores_bytes(const icm_ctx *ctx, const icm_db *db, size_t n_eyes,
  * fp16 CRT form keeps one byte per output residue and modulus). */
 icm_status icm_match_workspace_bytes(const icm_ctx *ctx, const icm_db *db, size_t n_eyes, icm_form form, size_t *bytes);
 
-/* Kernel launches that icm_match enqueues for n_eyes eyes in `form` on this chunk with the
- * context's current variant: 1 for the u64 and digit forms; for the CRT forms a product launch
- * and a recombination launch per column round (1,024 columns on the tcgen05 kernel, 512 on
- * mma.sync) and per group of limbs (the groups keep the residue scratch within 6 GiB); in the
+/* Kernel launches that icm_match enqueues on this chunk for a query of n_eyes eyes prepared in `form`
+ * and matched under the context's current variant: 1 for the u64 and digit forms; for the CRT forms
+ * a product launch and a recombination launch per column round (1,024 columns on the tcgen05 kernel,
+ * 512 on mma.sync) and per group of limbs (the groups keep the residue scratch within 6 GiB); in the
  * fp16 form on tcgen05 one more launch where the last columns (up to 64 past a multiple of 256) are
  * multiplied as digits instead of residues, and only that one if there are no others. */
 icm_status icm_match_launches(const icm_ctx *ctx, const icm_db *db, size_t n_eyes, icm_form form, size_t *n);
@@ -301,7 +301,10 @@ void icm_plan_destroy(icm_plan *plan);
  * 1 = free-running pairs; 2 = with a wave bound between pairs (a pair starts fetching its next tile
  * once every pair has fetched its current one; cooperative launch) and the moduli in groups of six;
  * 3 = with the wave bound and all moduli of a row tile side by side.  0 restores the default,
- * variant 2 (which the int8 form and odd K run as 256).  Results are identical; only speed differs. */
+ * variant 2 (which the int8 form and odd K run as 256).  Results are identical; only speed differs.
+ * Which columns are multiplied as digits instead of residues (icm_match_launches) is settled when a query
+ * is prepared, by the variant of that moment: such columns go to the tcgen05 digit kernel under a variant
+ * set later too, and a query prepared under 128 or 256 has none. */
 icm_status icm_ctx_set_variant(icm_ctx *ctx, int variant);
 /* Failure detection of the tcgen05 kernel (no counterpart in the paper).  Every device-side wait
  * of that kernel (barrier phases, the wave bound) gives up after wait_ns nanoseconds of

@@ -198,3 +198,26 @@ def test_ppmm_short_product_time():
             ts.append(a.elapsed_time(b))
         t[K] = min(ts)
     assert t[64] < 1.15 * t[63]
+
+
+@pytest.mark.parametrize("n_eyes", [1, 9, 40])
+def test_variant_set_after_preparation(rows, n_eyes):
+    """A query prepared under one variant gives the same residues under any other (its digit columns, if it has
+    some, stay with the digit kernel)."""
+    eng, W, dbs = rows
+    ct = eng.encrypt_query(W.q_codes[:n_eyes], W.q_masks[:n_eyes], W.eye_ids[:n_eyes])
+    res = []
+    try:
+        for prepare, match in [(256, 256), (2, 256), (2, 128), (2, 1), (256, 2), (256, 3)]:
+            C.icm_ctx_set_variant(eng.ctx, prepare)
+            q = eng.prepare(ct, n_eyes, "f16_crt")
+            C.icm_ctx_set_variant(eng.ctx, match)
+            outs = eng.match_batch(dbs, q)
+            torch.cuda.synchronize()
+            res.append([s.residues() for s in outs])
+    finally:
+        C.icm_ctx_set_variant(eng.ctx, 0)
+    C.icm_device_status(True)
+    for r in res[1:]:
+        for a, b in zip(r, res[0]):
+            assert np.array_equal(a, b)
