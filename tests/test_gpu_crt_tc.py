@@ -221,3 +221,29 @@ def test_variant_set_after_preparation(rows, n_eyes):
     for r in res[1:]:
         for a, b in zip(r, res[0]):
             assert np.array_equal(a, b)
+
+
+def test_digit_kernel_bounded_wait_runs_out(wide):
+    """The digit kernel's waits end by themselves: with a 20 ms bound and the query producers' copies withheld
+    (test-only switch) it records ICM_ETIMEOUT and returns, the status is then clear, and the next launch is
+    right."""
+    eng, W, dbs = wide
+    ct = eng.encrypt_query(W.q_codes[:1], W.q_masks[:1], W.eye_ids[:1])
+    q, ref = eng.prepare(ct, 1, "f16_crt"), eng.match(dbs[1], eng.prepare(ct, 1, "u64"))
+    assert C.icm_match_launches(eng.ctx, dbs[1].handle, 1, C.FORMS["f16_crt"]) == 1
+    torch.cuda.synchronize()
+    C.icm_device_status(True)
+    C.icm_ctx_set_device_wait(eng.ctx, 20_000_000, True)
+    try:
+        eng.match(dbs[1], q)
+        torch.cuda.synchronize()
+    finally:
+        C.icm_ctx_set_device_wait(eng.ctx, 0, False)
+    with pytest.raises(C.IcmError) as e:
+        C.icm_device_status(True)
+    assert e.value.status == C.ICM_ETIMEOUT
+    C.icm_device_status(True)
+    s = eng.match(dbs[1], q)
+    torch.cuda.synchronize()
+    C.icm_device_status(True)
+    assert np.array_equal(s.residues(), ref.residues())
