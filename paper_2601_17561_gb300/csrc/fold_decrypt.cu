@@ -267,8 +267,11 @@ __device__ __forceinline__ void rescale_one(const icm::RescaleConsts &k, const u
     }
 }
 
-// Two coefficients per thread (independent chains for latency hiding); consecutive threads read
-// consecutive words of a limb.
+// Two coefficients per thread, one after the other (36 registers hold one's words); consecutive threads read
+// consecutive words of a limb.  Bound by the waits on those loads (8 of the 18 cycles between two
+// instructions of a warp, 67% of the warps resident), with the FMA-heavy pipe 49% and DRAM 27% busy; so the
+// fewer products above gave 0.303 -> 0.277 ms for the rescaling and fold of 32 eyes x 3,000 codes on 8
+// limbs, and nothing at 1.3e8 coefficients (5.0 to 5.2 ms, 0.30 of the copy bandwidth).
 __global__ void __launch_bounds__(256) k_rescale(const __grid_constant__ RsArgs a) {
     const uint64_t c0 = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x);
     const uint64_t half = (a.n + 1) / 2;

@@ -1,9 +1,10 @@
 // Phase 1 of the fp16 small-modulus CRT product on the tcgen05 tensor cores (Blackwell 5th-gen
 // MMA with accumulators in tensor memory).  Same arithmetic as k_crt_p1<fp16> (ppmm_crt.cu):
 // for one (limb, database chunk, 128-row tile, modulus m_i, column round of up to 1,024) it computes
-// c_i = (sum_k a[k] b[k]) mod m_i over residues held exactly in fp16 (|r| <= 127), accumulating
-// in fp32 TMEM and reducing each accumulator modulo m_i every 1,024 columns of K so that it stays
-// an exact integer below 2^24 (odd moduli: 1024 * 127^2 + 128 < 2^24); c_i goes to the byte scratch
+// c_i = (sum_k a[k] b[k]) mod m_i over residues held exactly in fp16 (at most 128 in magnitude on the database
+// side, where the rounding of s / m may miss by less than 1 / m, and 127 on the query side), accumulating
+// in fp32 TMEM and reducing each accumulator modulo m_i (to a remainder below m_i <= 255 in magnitude) every
+// 1,024 columns of K, so that it stays an exact integer: 1024 * 128 * 127 + 254 < 2^24.  c_i goes to the byte scratch
 // that phase 2 (k_crt_combine) recombines.
 //
 // Tile of one block pair (a cluster of two on cta_group::2).  The queries are the M side and the
@@ -15,23 +16,15 @@
 // the database passes of a block that works alone on 128 x 512, with the same bytes of query
 // planes per MMA.  With fewer columns the accumulators are shared out to several moduli of the
 // same row tile (G column groups x NM moduli <= 4), which read one raw slab.
-//   What bounded the single-block form (563 cycles per 128 x 16 x 512 step against 256 of MMA): its
-//   conversions and copies.  The conversion took 11 half-rate integer instructions per two residues
-//   (res_pair: 9, three of them packed fp32).  A thread spends 51 cycles on a bulk copy that it
-//   issues inside a lane-dependent branch and 40 on a successful barrier probe, beside the
-//   converters' issue slots; copies of 4 to 16 KB took it ~383 cycles each, so one copy per 16-deep
-//   slab and producer cannot feed a 256-cycle slab, while L2 itself delivers 117 B/clk/SM to several
-//   threads.  Here an operand stage is 32 deep (one copy of up to 32 KB per modulus)
-//   and producers and issuer run on warp-uniform values with one elected lane.
+//   Copies: a bulk copy issued inside a lane-dependent branch takes a thread 51 cycles, an elected one 17, and
+//   one copy of 4 to 16 KB ~383 cycles, so an operand stage is 32 deep (one copy of up to 32 KB per
+//   modulus) and producers and issuer run on warp-uniform values with one elected lane.  Conversions:
+//   9 half-rate instructions per two residues (res_pair).
 //   The MMA runs at 71 cycles for M 256 N 128 K 16 (64 is the peak; N 256 reaches 128 of 128, but
 //   needs twice the conversions): 570 cycles per 32-deep stage.
 //   Measured (GB300): 32 eyes against N_db + 16,384 rows, 8 limbs: 218 -> 161 to 166 ms per pass; 734 cycles
 //   per stage at the 1.75 GHz that the power limit leaves.  What is left is the ring: 4 stages of
-//   36 KB, of which an accumulator under reduction holds up to two.  Tried on this form: an issuer
-//   thread per accumulator (four commits per stage: 26 ms where this takes 19.4), two issuers
-//   (19.9), stages of 16 k with 8 of them (23.6), the raw words loaded from global memory into the
-//   converters' registers one slab ahead, with 6 stages (26.8), 16 converter warps (11.2 for 10.1
-//   at 512 columns), moduli in groups of 3 / 9 instead of 6 (+1 / +3 %).
+//   36 KB, of which an accumulator under reduction holds up to two.
 //
 // Pipeline, the stages decoupled by rings of shared-memory slots with "full" / "empty" mbarriers:
 //  * raw producer (1 warp per block): one TMA load per 16-deep slab of the 64 x

@@ -6,8 +6,11 @@
 // products of a MAC (Karatsuba: the middle one is (a0 - a1)(b1 - b0), signed) go into three 64-bit
 // accumulators, one IMAD.WIDE each: S0 = sum a0 b0, D = sum (a0 - a1)(b1 - b0), S2 = sum a1 b1, and
 // S1 = sum a0 b1 + a1 b0 = S0 + S2 + D.  After 8 columns S0, S2 and |D| are below 2^63 and S1 is below
-// 2^64, so the sum modulo 2^64 is exact.  IMAD.WIDE (a half-rate instruction) bounds the kernel:
-// 4 eyes x 256 codes, 3 limbs, K = 20,480: 20.3 ms, 21.9 ms with the four products.  Every 8 columns the value
+// 2^64, so the sum modulo 2^64 is exact.  No one pipe bounds the kernel: the FMA-heavy pipe (IMAD.WIDE, a third
+// of the instructions) is 63% busy, the rest are the operands' loads and differences and the folds below, and
+// of the 5.0 cycles between two instructions of a warp (two warps per scheduler at 228 registers) 2.2
+// are waits on fixed latencies.  So a quarter fewer IMAD.WIDE gave only 7%: 4 eyes x 256 codes, 3 limbs,
+// K = 20,480: 20.3 ms, 21.9 ms with the four products.  Every 8 columns the value
 // S0 + S1 2^30 + S2 2^60 (< 2^125) is added into a 160-bit accumulator (a u128 and a carry word)
 // with integer adds and shifts, which issue on the ALU pipe while the IMAD.WIDE stream keeps the
 // FMA pipe busy.  The epilogue reduces the 160-bit sum modulo q_l with Shoup multiplications by
